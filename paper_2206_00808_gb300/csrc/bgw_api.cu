@@ -541,16 +541,13 @@ bgw::Axes mtxel_axes(const bgw_ctx_s *c, const QState &s, const int G0[3]) {
     return ax;
 }
 
-// Scratch of the matrix-element kernels for one k of q-point s (P = nv x nc
-// pairs, processed in batches of whole valence bands).
-cudaError_t ensure_mtxel_scratch(bgw_ctx_s *c, const QState &s, long P) {
+// Scratch of the matrix-element kernels for na x nb2 pairs of sphere s
+// (processed in batches of whole first-range bands).
+cudaError_t ensure_mtxel_scratch(bgw_ctx_s *c, const QState &s, int na, int nb2) {
     const long n01 = (long)c->box[0] * c->box[1];
     const int G0z[3] = {0, 0, 0};
     const bgw::Axes ax = mtxel_axes(c, s, G0z);
-    if (P > 0) {
-        const int nc = (int)(P / c->nv);
-        P = (long)bgw::mtxel_v_batch((int)(P / std::max(1, nc)), nc, ax, c->csize) * nc;
-    }
+    const long P = (long)bgw::mtxel_v_batch(na, nb2, ax, c->csize) * nb2;
     const long PA = bgw::mtxel_uses_a(ax) ? P : 0;
     cudaError_t e = c->A.ensure((size_t)(PA * n01 * s.w[2]) * c->csize, c->st);
     if (e == cudaSuccess) e = c->Bs.ensure((size_t)(P * c->box[0] * s.w[1] * s.w[2]) * c->csize, c->st);
@@ -706,7 +703,7 @@ cudaError_t ensure_chunk_scratch(bgw_ctx_s *c, const std::vector<QState> &qs, in
         const long P = (long)c->nv * s.nc;
         Pmax = std::max(Pmax, P);
         Mbytes = std::max(Mbytes, (long)kchunk * P * s.ng * (long)c->csize);
-        e = ensure_mtxel_scratch(c, s, P);
+        e = ensure_mtxel_scratch(c, s, c->nv, s.nc);
         if (e != cudaSuccess) return e;
     }
     const size_t mhalf = align256((size_t)Mbytes);
@@ -894,18 +891,6 @@ cudaError_t run_range(bgw_ctx_s *c, std::vector<QState> &qs, int nfreq, const do
 // ---- matrix elements of any band ranges (self-energy, BSE kernel) ----------
 namespace {
 
-// Scratch of the matrix-element kernels for na x nb2 pairs of sphere s.
-cudaError_t ensure_mtxel_scratch_pairs(bgw_ctx_s *c, const QState &s, int na, int nb2) {
-    const long n01 = (long)c->box[0] * c->box[1];
-    const int G0z[3] = {0, 0, 0};
-    const bgw::Axes ax = mtxel_axes(c, s, G0z);
-    const long P = (long)bgw::mtxel_v_batch(na, nb2, ax, c->csize) * nb2;
-    const long PA = bgw::mtxel_uses_a(ax) ? P : 0;
-    cudaError_t e = c->A.ensure((size_t)(PA * n01 * s.w[2]) * c->csize, c->st);
-    if (e == cudaSuccess) e = c->Bs.ensure((size_t)(P * c->box[0] * s.w[1] * s.w[2]) * c->csize, c->st);
-    return e;
-}
-
 // M[a][b][g] = M_{a0+a, b0+b}(k, q, G_g) for bands a0.. at k = kcrys[ik] and
 // b0.. at k + q (absolute band indices of the uploads) into the device
 // buffer M (row stride ng).  `clean` is cleared when the box aliases.
@@ -919,7 +904,7 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
     clean = clean && alias_free(c, ik, kp, G0, s);
     cudaError_t e = flush_k1(c);
     if (e != cudaSuccess) return c->cuda_fail(e, "deferred sphere-to-grid kernels");
-    e = ensure_mtxel_scratch_pairs(c, s, na, nb2);
+    e = ensure_mtxel_scratch(c, s, na, nb2);
     if (e != cudaSuccess) return c->cuda_fail(e, "matrix-element scratch");
     e = c->gmap_tmp.ensure(sizeof(int) * s.gmap.size(), c->st);
     if (e != cudaSuccess) return c->cuda_fail(e, "map buffer");
@@ -1256,10 +1241,9 @@ bgw_status bgw_mtxel_spinor(bgw_ctx c, const bgw_q *q, int ik, int v0, int nv, i
         return c->fail(BGW_E_STATE, "mtxel: k %d or its partner %d not uploaded", ik, kp);
     if (nv == 0 || nc == 0) return BGW_OK;
     const bool clean = alias_free(c, ik, kp, G0, s);
-    const long P = (long)nv * nc;
     cudaError_t e = flush_k1(c);
     if (e != cudaSuccess) return c->cuda_fail(e, "mtxel: deferred sphere-to-grid kernels");
-    e = ensure_mtxel_scratch(c, s, P);
+    e = ensure_mtxel_scratch(c, s, nv, nc);
     if (e != cudaSuccess) return c->cuda_fail(e, "mtxel: scratch");
     // The per-call map goes to a context buffer; reuse is stream-ordered and
     // a pageable-memory copy has read the host vector when the call returns.
