@@ -544,12 +544,11 @@ bgw::Axes mtxel_axes(const bgw_ctx_s *c, const QState &s, const int G0[3]) {
 // Scratch of the matrix-element kernels for na x nb2 pairs of sphere s
 // (processed in batches of whole first-range bands).
 cudaError_t ensure_mtxel_scratch(bgw_ctx_s *c, const QState &s, int na, int nb2) {
-    const long n01 = (long)c->box[0] * c->box[1];
     const int G0z[3] = {0, 0, 0};
     const bgw::Axes ax = mtxel_axes(c, s, G0z);
-    const long P = (long)bgw::mtxel_v_batch(na, nb2, ax, c->csize) * nb2;
-    const long PA = bgw::mtxel_uses_a(ax) ? P : 0;
-    cudaError_t e = c->A.ensure((size_t)(PA * n01 * s.w[2]) * c->csize, c->st);
+    const bool fixed = bgw::mtxel_fixed_point(ax, c->csize, c->mtxel_lanes);
+    const long P = (long)bgw::mtxel_v_batch(na, nb2, ax, c->csize, fixed) * nb2;
+    cudaError_t e = c->A.ensure(bgw::mtxel_a_bytes(na, nb2, ax, c->csize, fixed), c->st);
     if (e == cudaSuccess) e = c->Bs.ensure((size_t)(P * c->box[0] * s.w[1] * s.w[2]) * c->csize, c->st);
     return e;
 }
@@ -584,7 +583,8 @@ cudaError_t launch_mtxel(bgw_ctx_s *c, const QState &s, int ik, int kp, const in
     const int *gmap = static_cast<const int *>(s.gmap_dev.p);
     XProf xp(c);
     cudaError_t e = (c->prec == BGW_FP64)
-        ? bgw::mtxel_f64(Uv, Uc, nv, nc, ax, gmap, s.ng, c->A.p, c->Bs.p, M, ldm, c->st, 0, 0, c->mtxel_lanes, 0,
+        ? bgw::mtxel_f64(Uv, Uc, nv, nc, ax, gmap, s.ng, c->A.p, c->Bs.p, M, ldm, c->st, 0, 0, c->mtxel_lanes,
+                         bgw::mtxel_fixed_point(ax, c->csize, c->mtxel_lanes) ? bgw::kZyFixed : 0,
                          xp.get())
         : bgw::mtxel_f32(Uv, Uc, nv, nc, ax, gmap, s.ng, c->A.p, c->Bs.p, M, ldm, c->st, tv, tc, c->mtxel_lanes,
                          c->mtxel_zy, xp.get(), static_cast<int *>(c->errflag.p), c->test_drop_load == 2);
@@ -922,7 +922,8 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
     XProf xp(c);
     e = (c->prec == BGW_FP64)
             ? bgw::mtxel_f64(c->slot_ptr(sa, a0), c->slot_ptr(sb, b0), na, nb2, ax, gmap, s.ng, c->A.p, c->Bs.p, M,
-                             s.ng, c->st, 0, 0, c->mtxel_lanes, 0, xp.get())
+                             s.ng, c->st, 0, 0, c->mtxel_lanes,
+                         bgw::mtxel_fixed_point(ax, c->csize, c->mtxel_lanes) ? bgw::kZyFixed : 0, xp.get())
             : bgw::mtxel_f32(c->slot_ptr(sa, a0), c->slot_ptr(sb, b0), na, nb2, ax, gmap, s.ng, c->A.p, c->Bs.p, M,
                              s.ng, c->st, 0, 0, c->mtxel_lanes, c->mtxel_zy, xp.get(),
                              static_cast<int *>(c->errflag.p));

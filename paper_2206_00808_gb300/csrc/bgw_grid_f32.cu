@@ -2,6 +2,7 @@
 // (the mixed-precision path: complex64 grids and M).
 #define BGW_REAL float
 #define BGW_SUFFIX f32
+#define BGW_F32 1
 #include "bgw_grid_impl.cuh"
 
 namespace bgw {

@@ -2,7 +2,8 @@
 // arXiv:2206.00808 Sec. II), one template for FP64 and FP32.
 //
 // Included once per precision by bgw_grid_f64.cu / bgw_grid_f32.cu with
-// BGW_REAL and BGW_SUFFIX defined.
+// BGW_REAL and BGW_SUFFIX defined; BGW_GRID_PART 1 (sphere -> grid) or 2
+// (matrix elements) takes one half, so that the halves compile in parallel.
 //
 // Both 3-D transforms are done one axis at a time (one line per thread up to
 // N = 40; eight lanes per line through shared memory for cubic 48 and 64;
@@ -20,6 +21,12 @@
 // (f - s) mod N and the forward transform stores output f to slot
 // (f - s) mod N (see rot<N>).  Register indices stay compile-time.
 #pragma once
+#ifndef BGW_GRID_PART
+#define BGW_GRID_PART 0
+#endif
+#ifndef BGW_F32
+#define BGW_F32 0   // 1 in the FP32 translation unit: kernels that run in FP32 only
+#endif
 #include <cuda_pipeline.h>
 
 #include <cmath>
@@ -27,6 +34,7 @@
 
 #include "bgw_bounds.cuh"
 #include "bgw_fft.cuh"
+#include "bgw_fft_i64.cuh"
 #include "bgw_internal.h"
 #include "bgw_tc_common.cuh"
 
@@ -62,7 +70,12 @@ static cudaError_t upload_tables() {
             t32[off + j] = make_float2((float)c, (float)s);
         }
     }
+    int4 tq[kTwTotal];
+    int2 cq[kQcount];
+    fix_tables(tq, cq);
     cudaError_t e = cudaMemcpyToSymbol(c_tw64, t64, sizeof(double2) * kTwTotal);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_twq, tq, sizeof(int4) * kTwTotal);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_consq, cq, sizeof(int2) * kQcount);
     if (e != cudaSuccess) return e;
     return cudaMemcpyToSymbol(c_tw32, t32, sizeof(float2) * kTwTotal);
 }
@@ -76,6 +89,16 @@ template <int N>
 __device__ __forceinline__ int rot(int f, int ns) {
     const int j = f + ns;
     return j >= N ? j - N : j;
+}
+
+// One thread's line: FP32 in floating point, FP64 in 64-bit fixed point up
+// to the longest line whose integers fit a thread's registers (kFixMaxN).
+template <int S, int N>
+__device__ __forceinline__ void line_fft(C (&a)[N]) {
+    if constexpr (sizeof(T) == 8 && N <= kFixMaxN)
+        fft_line_fix<S, N>(a);
+    else
+        fft_line<T, S, N>(a);
 }
 
 // Kept outputs of a forward line whose cube starts at s: f = (s + j) mod N,
@@ -129,7 +152,7 @@ k1_xpass(const double2 *__restrict__ coeff, int ngw, long B, const int *__restri
         }
         a[f] = v;
     }
-    fft_line<T, +1, N>(a);
+    line_fft<+1, N>(a);
     C *out = S + b * N * yzs + yz;
 #pragma unroll
     for (int x = 0; x < N; ++x) out[x * yzs] = a[x];
@@ -150,7 +173,7 @@ k1_ypass(const C *__restrict__ S, long nbx, int w1, int w2, int s1, C *__restric
         const int j = rot<N>(f, ns);
         a[f] = (j < w1) ? S[(bx * w1 + j) * w2 + z] : C{T(0), T(0)};
     }
-    fft_line<T, +1, N>(a);
+    line_fft<+1, N>(a);
 #pragma unroll
     for (int y = 0; y < N; ++y) R[(bx * N + y) * w2 + z] = a[y];
 }
@@ -168,7 +191,7 @@ k1_zpass(const C *__restrict__ R, long nbxy, int w2, int s2, C *__restrict__ U) 
         const int j = rot<N>(f, ns);
         a[f] = (j < w2) ? R[t * w2 + j] : C{T(0), T(0)};
     }
-    fft_line<T, +1, N>(a);
+    line_fft<+1, N>(a);
 #pragma unroll
     for (int z = 0; z < N; ++z) U[t * N + z] = a[z];
 }
@@ -195,7 +218,7 @@ k2_zpass(const C *__restrict__ Uv, const C *__restrict__ Uc, int nc, long P, lon
 #pragma unroll
     for (int z = 0; z < N; ++z)
         a[z] = rho2(v0[z], c0[z], v0[vol + z], c0[vol + z]);
-    fft_line<T, -1, N>(a);
+    line_fft<-1, N>(a);
     store_kept<N, WIN>(a, A + (p * plane + xy) * w2, 1, N - s2, w2);
 }
 
@@ -210,7 +233,7 @@ k2_ypass(const C *__restrict__ A, long npx, int w1, int w2, int s1, C *__restric
     C a[N];
 #pragma unroll
     for (int y = 0; y < N; ++y) a[y] = A[(px * N + y) * w2 + jz];
-    fft_line<T, -1, N>(a);
+    line_fft<-1, N>(a);
     store_kept<N, WIN>(a, Bs + px * w1 * w2 + jz, w2, N - s1, w1);
 }
 
@@ -235,7 +258,7 @@ k2_xpass_gather(const C *__restrict__ Bs, long P, int PP, int w0, int w1, int w2
         C a[N];
 #pragma unroll
         for (int x = 0; x < N; ++x) a[x] = bi[x * lines];
-        fft_line<T, -1, N>(a);
+        line_fft<-1, N>(a);
         store_kept<N, WIN>(a, cube + pp * csz + ll, lines, ns, w0);
     }
     __syncthreads();
@@ -273,7 +296,7 @@ k2_xpass_scatter(const C *__restrict__ Bs, long P, int w0, int w1, int w2, int s
     C a[N];
 #pragma unroll
     for (int x = 0; x < N; ++x) a[x] = Bs[(p * N + x) * lines + l];
-    fft_line<T, -1, N>(a);
+    line_fft<-1, N>(a);
     const int ns = N - s0;
 #pragma unroll
     for (int f = 0; f < N; ++f) {
@@ -641,7 +664,7 @@ __device__ __forceinline__ void k1_fused_body(const double2 *__restrict__ cb, in
                 a[f] = v;
             }
         }
-        fft_line<T, +1, N>(a);
+        line_fft<+1, N>(a);
 #pragma unroll
         for (int x = 0; x < N; ++x) X[x * yzs + l] = a[x];
     }
@@ -657,7 +680,7 @@ __device__ __forceinline__ void k1_fused_body(const double2 *__restrict__ cb, in
                 const int j = rot<N>(f, ns1);
                 a[f] = (j < w1) ? xi[j * w2] : C{T(0), T(0)};
             }
-            fft_line<T, +1, N>(a);
+            line_fft<+1, N>(a);
             C *yo = Y + xl * N * w2p + z;
 #pragma unroll
             for (int y = 0; y < N; ++y) yo[y * w2p] = a[y];
@@ -672,7 +695,7 @@ __device__ __forceinline__ void k1_fused_body(const double2 *__restrict__ cb, in
                 const int j = rot<N>(f, ns2);
                 a[f] = (j < w2) ? yi[j] : C{T(0), T(0)};
             }
-            fft_line<T, +1, N>(a);
+            line_fft<+1, N>(a);
             C *o = out + ((long)(x0 + xl) * N + y) * N;
             if constexpr (sizeof(T) == 4 && N % 2 == 0) {
 #pragma unroll
@@ -838,7 +861,7 @@ k2_zy_plane(const C *__restrict__ Uv, const C *__restrict__ Uc, int nv, int nc, 
 #pragma unroll
             for (int z = 0; z < N; ++z) a[z] = rho2(pv[z], pc[z], pv[PS + z], pc[PS + z]);
         }
-        fft_line<T, -1, N>(a);
+        line_fft<-1, N>(a);
         store_kept<N, WIN>(a, Z + ((long)pr * N + y) * w2, 1, ns2, w2);
     }
     __syncthreads();
@@ -850,7 +873,7 @@ k2_zy_plane(const C *__restrict__ Uv, const C *__restrict__ Uc, int nv, int nc, 
         C a[N];
 #pragma unroll
         for (int y = 0; y < N; ++y) a[y] = zi[y * w2];
-        fft_line<T, -1, N>(a);
+        line_fft<-1, N>(a);
         const long p = (long)(v0 + v) * nc + (c0 + c);
         store_kept<N, WIN>(a, Bs + ((p * n0 + x) * w1) * w2 + jz, w2, ns1, w1);
     }
@@ -1007,7 +1030,7 @@ k2_zy_stream(const C *__restrict__ Uv, const C *__restrict__ Uc, int nv, int nc,
                     a[2 * z] = rho2(C{va.x, va.y}, C{ca.x, ca.y}, C{vb.x, vb.y}, C{cb.x, cb.y});
                     a[2 * z + 1] = rho2(C{va.z, va.w}, C{ca.z, ca.w}, C{vb.z, vb.w}, C{cb.z, cb.w});
                 }
-                fft_line<T, -1, N>(a);
+                line_fft<-1, N>(a);
                 store_kept<N, WIN>(a, Z0 + (k & 1) * ZS + ((long)pr * N + y) * w2, 1, ns2, w2);
             }
         } else if (k >= 1) {
@@ -1022,7 +1045,7 @@ k2_zy_stream(const C *__restrict__ Uv, const C *__restrict__ Uc, int nv, int nc,
                 C b[N];
 #pragma unroll
                 for (int yy = 0; yy < N; ++yy) b[yy] = zi[yy * w2];
-                fft_line<T, -1, N>(b);
+                line_fft<-1, N>(b);
                 const long p = (long)(v0 + v) * nc + (c0 + c);
                 store_kept<N, WIN>(b, Bs + ((p * n0 + x) * w1) * w2 + jz, w2, ns1, w1);
             }
@@ -1076,7 +1099,7 @@ k1_yz_plane(const C *__restrict__ S, long B, int TB, int w1, int w2, int s1, int
             const int j = rot<N>(f, ns1);
             a[f] = (j < w1) ? in[(b * w1 + j) * w2 + z] : C{T(0), T(0)};
         }
-        fft_line<T, +1, N>(a);
+        line_fft<+1, N>(a);
 #pragma unroll
         for (int y = 0; y < N; ++y) P[(b * N + y) * PW + z] = a[y];
     }
@@ -1089,7 +1112,7 @@ k1_yz_plane(const C *__restrict__ S, long B, int TB, int w1, int w2, int s1, int
             const int j = rot<N>(f, ns2);
             a[f] = (j < w2) ? P[(b * N + y) * PW + j] : C{T(0), T(0)};
         }
-        fft_line<T, +1, N>(a);
+        line_fft<+1, N>(a);
         C *o = out + ((long)b * N + y) * (N + 1);
 #pragma unroll
         for (int z = 0; z < N; ++z) o[z] = a[z];
@@ -1159,6 +1182,21 @@ static inline unsigned quads_for(long lines) { return (unsigned)((4 * lines + kL
         default: return cudaErrorInvalidValue;                                        \
     }
 
+#if BGW_GRID_PART != 2   // sphere -> grid
+static cudaError_t launch_fused_batch(const K1Batch &jb, int n, size_t smem, cudaStream_t st) {
+    BGW_FOR_EACH_LEN(n, {
+        if constexpr (N < kCoopMinN) {
+            if (smem > 48 * 1024) {
+                const cudaError_t e = cudaFuncSetAttribute(k1_fused_batch<N>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return e;
+            }
+            k1_fused_batch<N><<<(unsigned)(jb.njobs * jb.B), kFusedThreads, smem, st>>>(jb);
+        }
+    });
+    return cudaGetLastError();
+}
+
 static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *cube_map,
                                const Axes &a, void *S, void *R, void *U, cudaStream_t st, int path) {
     const long nb = B;
@@ -1166,7 +1204,8 @@ static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *c
     const double2 *cf = reinterpret_cast<const double2 *>(coeff);
     const int *inv = cube_map + (long)a.w[0] * a.w[1] * a.w[2];
     bool oct = oct_len(a) && (path == 3 || (use_coop(a) && use_oct(a)));
-    if (path == 4 && sizeof(T) == 4 && a.n[0] == a.n[1] && a.n[1] == a.n[2] && a.n[0] < kCoopMinN) {
+#if BGW_F32
+    if (path == 4 && a.n[0] == a.n[1] && a.n[1] == a.n[2] && a.n[0] < kCoopMinN) {
         // cube-less one-kernel transform, three CTAs per SM, where it fits
         int KP = 0;
         for (int chunks = 1; chunks <= a.n[0] && !KP; ++chunks) {
@@ -1190,11 +1229,13 @@ static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *c
             return cudaGetLastError();
         }
     }
+#endif
     const int KP = (path == 1 || oct) ? 0 : fused_planes(a, path == 2 ? kFusedSmemMax : kFusedSmemAuto);
     // automatic choice for cubic FP32 boxes of 32 and 40 whose x-transformed
     // cube does not fit the one-kernel transform: the eight-lane kernels
     // (GaSb-like 32^3: 48.8 -> 41.4 ms per q-point against the one-lane passes)
     if (path == 0 && !KP && sizeof(T) == 4 && oct_len(a)) oct = true;
+#if BGW_F32
     if (KP) {
         const size_t smem = fused_smem(a, KP);
         cudaError_t e = cudaSuccess;
@@ -1211,6 +1252,15 @@ static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *c
         });
         return cudaGetLastError();
     }
+#else
+    if (KP) {
+        K1Batch jb;
+        jb.njobs = 1;
+        jb.B = B;
+        jb.job[0] = K1BatchJob{cf, inv, Up, ngw, a.w[0], a.w[1], a.w[2], a.s[0], a.s[1], a.s[2], KP};
+        return launch_fused_batch(jb, a.n[0], fused_smem(a, KP), st);
+    }
+#endif
     if (oct) {
         const long groups = nb * a.w[1] * a.w[2];
         BGW_FOR_EACH_OCT_LEN(a.n[0], (k1_xpass_oct<N><<<(unsigned)((groups + 31) / 32), kOctThreads, 0, st>>>(
@@ -1233,6 +1283,7 @@ static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *c
         BGW_FOR_EACH_LEN(a.n[0], (k1_xpass<N><<<blocks_for(lines), kLineThreads, 0, st>>>(
                                      cf, ngw, nb, cube_map, a.w[0], a.w[1], a.w[2], a.s[0], Sp)));
     }
+#if BGW_F32
     if (use_plane_kernels(a)) {
         const int n = a.n[1];
         auto yz_smem = [&](int tb) {
@@ -1259,6 +1310,7 @@ static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *c
             return cudaGetLastError();
         }
     }
+#endif
     {
         const long nbx = nb * a.n[0];
         BGW_FOR_EACH_LEN(a.n[1], (k1_ypass<N><<<blocks_for(nbx * a.w[2]), kLineThreads, 0, st>>>(
@@ -1310,23 +1362,15 @@ static cudaError_t wfn_to_grid_batch(const K1Job *jobs, int n, int B, cudaStream
             d.s2 = j.a.s[2];
             d.KP = fused_planes(j.a, kFusedSmemAuto);
         }
-        BGW_FOR_EACH_LEN(N0, {
-            if constexpr (N < kCoopMinN) {
-                if (smem > 48 * 1024) {
-                    e = cudaFuncSetAttribute(k1_fused_batch<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-                    if (e != cudaSuccess) return e;
-                }
-                k1_fused_batch<N><<<(unsigned)(jb.njobs * B), kFusedThreads, smem, st>>>(jb);
-            }
-        });
-        e = cudaGetLastError();
+        e = launch_fused_batch(jb, N0, smem, st);
         if (e != cudaSuccess) return e;
     }
     *batched = true;
     return cudaSuccess;
 }
 
+#endif
+#if BGW_GRID_PART != 1   // matrix elements
 // Pair tiles (TV valence x TC conduction) of the plane kernel that fit
 // kPlaneSmemMax, best first: least staged data per pair, then most pairs.
 static size_t plane_smem(int tv, int tc, int n, int w2) {
@@ -1402,8 +1446,7 @@ static cudaError_t xpass(const C *Bp, long P, const Axes &a, const int *gmap, in
     BGW_FOR_EACH_LEN(a.n[0], {
         const int PP = gather_pairs(a, P);
         auto kern = k2_xpass_gather<N, false>;
-        if constexpr (N > 2 * kWin + 1)
-            if (kept_in_window(a, 0)) kern = k2_xpass_gather<N, true>;
+        if (kept_in_window(a, 0)) kern = k2_xpass_gather<N, (N > 2 * kWin + 1)>;
         if (smem * PP > 48 * 1024) {
             e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem * PP));
             if (e != cudaSuccess) return e;
@@ -1502,8 +1545,7 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
         BGW_FOR_EACH_LEN(a.n[0], {
             const int PP = gather_pairs(a, P);
             auto kern = k2_xpass_gather<N, false>;
-            if constexpr (N > 2 * kWin + 1)
-                if (kept_in_window(a, 0)) kern = k2_xpass_gather<N, true>;
+            if (kept_in_window(a, 0)) kern = k2_xpass_gather<N, (N > 2 * kWin + 1)>;
             if (smem * PP > 48 * 1024) {
                 e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem * PP));
                 if (e != cudaSuccess) return e;
@@ -1513,6 +1555,7 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
         });
         return cudaGetLastError();
     }
+#if BGW_F32
     if ((zy == 2 || (zy == 0 && tv_req <= 0)) && use_stream(a)) {
         // streamed pair density + z + y: conduction ranges sized for about four
         // waves of one CTA per SM
@@ -1572,6 +1615,15 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
         XMark xm(hook, 1);
         return xpass(Bp, P, a, gmap, ng, Mp, ldm, st);
     }
+#endif
+#if !BGW_F32
+    if (zy == kZyFixed) {
+        const cudaError_t e = mtxel_zy_fix(uv, uc, nv, nc, a, Ap, Bp, st);
+        if (e != cudaSuccess) return e;
+        XMark xm(hook, 3);
+        return xpass(Bp, P, a, gmap, ng, Mp, ldm, st);
+    }
+#endif
     int TV = 0, TC = 0;
     if (use_plane_kernels(a)) {
         if (tv_req > 0 && tc_req > 0 && plane_smem(tv_req, tc_req, a.n[1], a.w[2]) <= kPlaneSmemLarge) {
@@ -1596,6 +1648,7 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
                                           Bp, P, a.w[0], a.w[1], a.w[2], a.s[0], gmap + ng, scale, Mp, ldm)));
         return cudaGetLastError();
     }
+#if BGW_F32
     if (TV > 0) {
         dim3 grid((unsigned)a.n[0], (unsigned)((nv + TV - 1) / TV), (unsigned)((nc + TC - 1) / TC));
         cudaError_t e = cudaSuccess;
@@ -1622,20 +1675,20 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
             kern<<<grid, large ? kPlaneThreadsLarge : kPlaneThreads, psmem, st>>>(
                 uv, uc, nv, nc, TV, TC, a.w[1], a.w[2], a.s[1], a.s[2], Bp);
         });
-    } else {
+    } else
+#endif
+    {
         const long plane = (long)a.n[0] * a.n[1];
         const bool wz = kept_in_window(a, 2), wy = kept_in_window(a, 1);
         BGW_FOR_EACH_LEN(a.n[2], {
             auto kern = k2_zpass<N, false>;
-            if constexpr (N > 2 * kWin + 1)
-                if (wz) kern = k2_zpass<N, true>;
+            if (wz) kern = k2_zpass<N, (N > 2 * kWin + 1)>;
             kern<<<blocks_for(P * plane), kLineThreads, 0, st>>>(uv, uc, nc, P, plane, a.w[2], a.s[2], Ap);
         });
         const long npx = P * a.n[0];
         BGW_FOR_EACH_LEN(a.n[1], {
             auto kern = k2_ypass<N, false>;
-            if constexpr (N > 2 * kWin + 1)
-                if (wy) kern = k2_ypass<N, true>;
+            if (wy) kern = k2_ypass<N, (N > 2 * kWin + 1)>;
             kern<<<blocks_for(npx * a.w[2]), kLineThreads, 0, st>>>(Ap, npx, a.w[1], a.w[2], a.s[1], Bp);
         });
     }
@@ -1651,7 +1704,7 @@ static cudaError_t mtxel(const void *Uv, const void *Uc, int nv, int nc, const A
     const C *uv = static_cast<const C *>(Uv), *uc = static_cast<const C *>(Uc);
     C *Ap = static_cast<C *>(A), *Bp = static_cast<C *>(Bs), *Mp = static_cast<C *>(M);
     const long vol = (long)a.n[0] * a.n[1] * a.n[2];
-    const int VB = mtxel_v_batch(nv, nc, a, sizeof(C));
+    const int VB = mtxel_v_batch(nv, nc, a, sizeof(C), sizeof(T) == 8 && zy == kZyFixed);
     for (int vb0 = 0; vb0 < nv; vb0 += VB) {
         const int nvb = nv - vb0 < VB ? nv - vb0 : VB;
         cudaError_t e = mtxel_batch(uv + (long)vb0 * 2 * vol, uc, nvb, nc, a, gmap, ng, Ap, Bp,
@@ -1660,6 +1713,8 @@ static cudaError_t mtxel(const void *Uv, const void *Uc, int nv, int nc, const A
     }
     return cudaSuccess;
 }
+
+#endif
 
 #undef BGW_FOR_EACH_LEN
 #undef BGW_FOR_EACH_COOP_LEN

@@ -62,6 +62,8 @@ cudaError_t wfn_to_grid_batch_f32(const K1Job *jobs, int n, int B, cudaStream_t 
 // N = 32, 40, 48 or 64 (automatic choice uses them for 48 and 64 only).
 // Pairs are processed in batches of mtxel_v_batch(...) valence bands x nc, so
 // A and Bs need room for that many pairs only.
+// zy (FP64): kZyFixed takes the fixed-point z + y kernel (the caller checked
+// mtxel_fixed_point and sized A by mtxel_a_bytes), else the FP64 passes.
 // zy (FP32): 0 automatic (the streamed z + y kernel where it applies, unless a
 // pair tile tv x tc is given), 1 the plane kernel with the pair tile tv x tc,
 // 2 streamed where it applies.
@@ -75,6 +77,7 @@ struct XPassHook {
     void (*fn)(void *ctx, int begin, int kernels);
     void *ctx;
 };
+constexpr int kZyFixed = 3;
 cudaError_t mtxel_f64(const void *Uv, const void *Uc, int nv, int nc, const Axes &a,
                       const int *gmap, int ng, void *A, void *Bs, void *M, long ldm,
                       cudaStream_t st, int tv = 0, int tc = 0, int lanes = 0, int zy = 0,
@@ -113,14 +116,33 @@ inline bool wfn_uses_r(const Axes &a, size_t csize) {
     return !fp32_square;
 }
 
+// Whether the FP64 matrix elements of a context take the fixed-point z + y
+// kernel (bgw_zy_fix.cu): square y-z planes whose lines fit one thread, unless
+// the eight-lane kernels are asked for.  (bgw_mtxel_spinor_noalloc keeps the
+// FP64 pair density: its grids come from the caller, and one scale per plane
+// is as exact as FP64 only for grids that carry the rounding of a transform.)
+inline bool mtxel_fixed_point(const Axes &a, size_t csize, int lanes) {
+    const bool cubic = a.n[0] == a.n[1] && a.n[1] == a.n[2];
+    return csize == 16 && a.n[1] == a.n[2] && a.n[1] <= 40 && !(lanes == 8 && cubic && (a.n[0] == 32 || a.n[0] == 40));
+}
+// Bands of each side that kernel holds as integers at a time: up to 1 GiB in all.
+inline void fix_band_caps(const Axes &a, int nv, int nc, int *vcap, int *ccap) {
+    const size_t band = (size_t)a.n[0] * (2 * 16 * (size_t)a.n[1] * a.n[2] + sizeof(int));
+    const size_t half = ((size_t)1 << 29) / band;
+    const int cap = half < 1 ? 1 : half > (1u << 20) ? 1 << 20 : (int)half;
+    *vcap = nv < cap ? nv : cap;
+    *ccap = nc < cap ? nc : cap;
+}
+
 // Valence bands per batch of the matrix-element kernels: their scratch
-// (A, where used, + Bs per pair) stays under 1 GiB.  When the bands need more
-// than one batch, a batch is a whole number of the streamed FP32 kernel's
-// valence groups (5 bands at N = 24, else 4), so no batch but the last ends
-// in a short group (18 bands ran as 17 + 1: groups 4,4,4,4,1 and 1).
-inline int mtxel_v_batch(int nv, int nc, const Axes &a, size_t csize) {
+// (A, where it holds pairs, + Bs per pair) stays under 1 GiB.  When the bands
+// need more than one batch, a batch is a whole number of the streamed FP32
+// kernel's valence groups (5 bands at N = 24, else 4), so no batch but the last
+// ends in a short group (18 bands ran as 17 + 1: groups 4,4,4,4,1 and 1).
+inline int mtxel_v_batch(int nv, int nc, const Axes &a, size_t csize, bool fixed) {
+    const bool pairs_in_a = mtxel_uses_a(a) && !fixed;
     const size_t per_pair =
-        csize * ((mtxel_uses_a(a) ? (size_t)a.n[0] * a.n[1] * a.w[2] : 0) + (size_t)a.n[0] * a.w[1] * a.w[2]);
+        csize * ((pairs_in_a ? (size_t)a.n[0] * a.n[1] * a.w[2] : 0) + (size_t)a.n[0] * a.w[1] * a.w[2]);
     const size_t cap = (size_t)1 << 30;
     size_t vb = cap / (per_pair * (size_t)(nc > 0 ? nc : 1) + 1);
     if (vb < 1) vb = 1;
@@ -129,6 +151,22 @@ inline int mtxel_v_batch(int nv, int nc, const Axes &a, size_t csize) {
     if (vb >= group) vb -= vb % group;
     return (int)vb;
 }
+// Bytes of scratch A for one such batch: the z-pass output of its pairs, or the
+// bands of the fixed-point kernel.
+inline size_t mtxel_a_bytes(int nv, int nc, const Axes &a, size_t csize, bool fixed) {
+    const int vb = mtxel_v_batch(nv, nc, a, csize, fixed);
+    if (fixed) {
+        int vcap, ccap;
+        fix_band_caps(a, vb, nc, &vcap, &ccap);
+        return (size_t)(vcap + ccap) * a.n[0] * (2 * 16 * (size_t)a.n[1] * a.n[2] + sizeof(int));
+    }
+    return mtxel_uses_a(a) ? (size_t)vb * nc * a.n[0] * a.n[1] * a.w[2] * csize : 0;
+}
+// z + y passes of nv x nc pairs into Bs (see mtxel_f64), FP64 through 64-bit
+// fixed point; ws: mtxel_a_bytes of scratch.
+cudaError_t zy_fix_tables_init();
+cudaError_t mtxel_zy_fix(const void *Uv, const void *Uc, int nv, int nc, const Axes &a, void *ws, void *Bs,
+                         cudaStream_t st);
 
 // Candidate pair tiles (tv, tc) of the plane-fused FP32 kernel for this shape,
 // best first by the staging heuristic; returns how many were written.

@@ -136,7 +136,7 @@ extern "C" bgw_status bgw_mtxel_spinor_noalloc(const int fft[3], const void *Uv,
     const size_t a_pair = bgw::mtxel_uses_a(ax) ? (size_t)fft[0] * fft[1] * ax.w[2] * 16 : 0;
     const size_t b_pair = (size_t)fft[0] * ax.w[1] * ax.w[2] * 16;
     auto need = [&](long vb) {
-        const long pb = (long)std::min(vb, (long)bgw::mtxel_v_batch((int)vb, nc, ax, 16)) * nc;
+        const long pb = (long)std::min(vb, (long)bgw::mtxel_v_batch((int)vb, nc, ax, 16, false)) * nc;
         return gbytes + round_up((size_t)pb * a_pair) + round_up((size_t)pb * b_pair);
     };
     const size_t cap = (size_t)BGW_NOALLOC_SCRATCH_BYTES;
@@ -180,7 +180,7 @@ extern "C" bgw_status bgw_mtxel_spinor_noalloc(const int fft[3], const void *Uv,
     }
     char *base = static_cast<char *>(scratch);
     int *gmap = reinterpret_cast<int *>(base);
-    const long pb = (long)std::min(vb, (long)bgw::mtxel_v_batch((int)vb, nc, ax, 16)) * nc;
+    const long pb = (long)std::min(vb, (long)bgw::mtxel_v_batch((int)vb, nc, ax, 16, false)) * nc;
     char *abuf = base + gbytes;
     char *bbuf = abuf + round_up((size_t)pb * a_pair);
     // pageable source: the copy waits for earlier work on the stream and has
