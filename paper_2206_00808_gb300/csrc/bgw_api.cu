@@ -274,6 +274,13 @@ struct bgw_ctx_s {
         return e == cudaErrorMemoryAllocation ? BGW_E_NOMEM : BGW_E_CUDA;
     }
     long grid_elems_per_k() const { return (long)nb * 2 * nbox; }
+    // FP64 contexts whose grids are integer grids (bgw_internal.h): the scales
+    // [slot][band][N1] follow the grids in the same allocation
+    bool fixed = false;
+    int *scale_ptr(int slot, int band) {
+        return reinterpret_cast<int *>(static_cast<char *>(grids.p) + (size_t)nslots * grid_elems_per_k() * csize) +
+               ((long)slot * nb + band) * box[0];
+    }
     char *slot_ptr(int slot, int band) {
         return static_cast<char *>(grids.p) + ((long)slot * grid_elems_per_k() + (long)band * 2 * nbox) * csize;
     }
@@ -298,7 +305,8 @@ cudaError_t ensure_slots(bgw_ctx_s *c) {
     if (c->nslots > 0) return cudaSuccess;
     const int n = (c->grid_slots_opt > 0 && c->grid_slots_opt < c->nk) ? std::max(2, c->grid_slots_opt)
                                                                          : c->nk;
-    cudaError_t e = c->grids.ensure((size_t)n * c->grid_elems_per_k() * c->csize, c->st);
+    const size_t scales = c->fixed ? sizeof(int) * (size_t)n * c->nb * c->box[0] : 0;
+    cudaError_t e = c->grids.ensure((size_t)n * c->grid_elems_per_k() * c->csize + scales, c->st);
     if (e != cudaSuccess) return e;
     c->nslots = n;
     c->slot_k.assign(n, -1);
@@ -319,18 +327,25 @@ cudaError_t run_k1(bgw_ctx_s *c, int ik, const double *src, int slot) {
         ax.w[a] = w[a];
         ax.s[a] = pmod(kp.lo[a], c->box[a]);
     }
+    // integer grids straight from the coefficients, or, where a kernel path is
+    // asked for, through an FP64 grid
+    const bool direct = c->fixed && c->k1_path == 0;
     const size_t rbytes =
-        bgw::wfn_uses_r(ax, c->csize) ? (size_t)B * c->box[0] * c->box[1] * w[2] * c->csize : 0;
+        !direct && bgw::wfn_uses_r(ax, c->csize) ? (size_t)B * c->box[0] * c->box[1] * w[2] * c->csize : 0;
     cudaError_t e = c->S.ensure(sbytes, c->st);
     if (e == cudaSuccess) e = c->R.ensure(rbytes, c->st);
     if (e != cudaSuccess) return e;
     void *U = c->slot_ptr(slot, 0);
     const int *mp = static_cast<const int *>(kp.map_dev.p);
     const int rec = c->stage_begin(0);
+    if (direct)
+        e = bgw::wfn_to_fix(src, kp.ngw, c->nb, mp, ax, c->S.p, U, c->scale_ptr(slot, 0), c->st);
+    else
     e = (c->prec == BGW_FP64)
             ? bgw::wfn_to_grid_f64(src, kp.ngw, (int)B, mp, ax, c->S.p, c->R.p, U, c->st, c->k1_path)
             : bgw::wfn_to_grid_f32(src, kp.ngw, (int)B, mp, ax, c->S.p, c->R.p, U, c->st, c->k1_path);
-    c->stage_end(rec, 3);
+    if (e == cudaSuccess && c->fixed && !direct) e = bgw::grid_to_fix(U, c->nb, ax, c->scale_ptr(slot, 0), c->st);
+    c->stage_end(rec, direct ? 2 : 3);
     return e;
 }
 
@@ -420,7 +435,7 @@ cudaError_t flush_k1(bgw_ctx_s *c) {
     }
     if (e != cudaSuccess) return e;
     bool batched = false;
-    if (c->k1_path == 0) {
+    if (c->k1_path == 0 && !c->fixed) {
         const int rec = c->stage_begin(0);
         const int B = 2 * c->nb;
         e = (c->prec == BGW_FP64) ? bgw::wfn_to_grid_batch_f64(jobs.data(), (int)jobs.size(), B, c->st, &batched)
@@ -546,9 +561,11 @@ bgw::Axes mtxel_axes(const bgw_ctx_s *c, const QState &s, const int G0[3]) {
 cudaError_t ensure_mtxel_scratch(bgw_ctx_s *c, const QState &s, int na, int nb2) {
     const int G0z[3] = {0, 0, 0};
     const bgw::Axes ax = mtxel_axes(c, s, G0z);
-    const bool fixed = bgw::mtxel_fixed_point(ax, c->csize, c->mtxel_lanes);
+    const bool eight = c->fixed && bgw::mtxel_eight_lanes(ax.n, c->mtxel_lanes);   // FP64 copies of the bands in A
+    const bool fixed = c->fixed && !eight;
     const long P = (long)bgw::mtxel_v_batch(na, nb2, ax, c->csize, fixed) * nb2;
-    cudaError_t e = c->A.ensure(bgw::mtxel_a_bytes(na, nb2, ax, c->csize, fixed), c->st);
+    cudaError_t e = c->A.ensure(eight ? (size_t)(na + nb2) * 2 * c->nbox * c->csize
+                                      : bgw::mtxel_a_bytes(na, nb2, ax, c->csize, fixed), c->st);
     if (e == cudaSuccess) e = c->Bs.ensure((size_t)(P * c->box[0] * s.w[1] * s.w[2]) * c->csize, c->st);
     return e;
 }
@@ -570,6 +587,27 @@ struct XProf {
     }
 };
 
+// FP64 matrix elements of bands a0.. in slot sa with bands b0.. in slot sb.
+cudaError_t mtxel_f64_bands(bgw_ctx_s *c, const bgw::Axes &ax, int sa, int a0, int na, int sb, int b0, int nb2,
+                            const int *gmap, int ng, void *M, long ldm, const bgw::XPassHook *hook) {
+    const void *ua = c->slot_ptr(sa, a0), *ub = c->slot_ptr(sb, b0);
+    const int *ga = nullptr, *gb = nullptr;
+    if (c->fixed) {
+        ga = c->scale_ptr(sa, a0);
+        gb = c->scale_ptr(sb, b0);
+        if (bgw::mtxel_eight_lanes(ax.n, c->mtxel_lanes)) {
+            char *fa = static_cast<char *>(c->A.p), *fb = fa + (size_t)na * 2 * c->nbox * c->csize;
+            cudaError_t e = bgw::fix_to_grid(ua, ga, na, ax, fa, c->st);
+            if (e == cudaSuccess) e = bgw::fix_to_grid(ub, gb, nb2, ax, fb, c->st);
+            if (e != cudaSuccess) return e;
+            ua = fa;
+            ub = fb;
+            ga = gb = nullptr;
+        }
+    }
+    return bgw::mtxel_f64(ua, ub, na, nb2, ax, gmap, ng, c->A.p, c->Bs.p, M, ldm, c->st, c->mtxel_lanes, hook, ga, gb);
+}
+
 cudaError_t launch_mtxel(bgw_ctx_s *c, const QState &s, int ik, int kp, const int G0[3], int v0,
                          int nv, int c0, int nc, void *M, long ldm, int tv = 0, int tc = 0) {
     const bgw::Axes ax = mtxel_axes(c, s, G0);
@@ -583,9 +621,7 @@ cudaError_t launch_mtxel(bgw_ctx_s *c, const QState &s, int ik, int kp, const in
     const int *gmap = static_cast<const int *>(s.gmap_dev.p);
     XProf xp(c);
     cudaError_t e = (c->prec == BGW_FP64)
-        ? bgw::mtxel_f64(Uv, Uc, nv, nc, ax, gmap, s.ng, c->A.p, c->Bs.p, M, ldm, c->st, 0, 0, c->mtxel_lanes,
-                         bgw::mtxel_fixed_point(ax, c->csize, c->mtxel_lanes) ? bgw::kZyFixed : 0,
-                         xp.get())
+        ? mtxel_f64_bands(c, ax, sv, v0, nv, sc, c->nv + c0, nc, gmap, s.ng, M, ldm, xp.get())
         : bgw::mtxel_f32(Uv, Uc, nv, nc, ax, gmap, s.ng, c->A.p, c->Bs.p, M, ldm, c->st, tv, tc, c->mtxel_lanes,
                          c->mtxel_zy, xp.get(), static_cast<int *>(c->errflag.p), c->test_drop_load == 2);
     xp.finish();
@@ -921,9 +957,7 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
     const int *gmap = static_cast<const int *>(c->gmap_tmp.p);
     XProf xp(c);
     e = (c->prec == BGW_FP64)
-            ? bgw::mtxel_f64(c->slot_ptr(sa, a0), c->slot_ptr(sb, b0), na, nb2, ax, gmap, s.ng, c->A.p, c->Bs.p, M,
-                             s.ng, c->st, 0, 0, c->mtxel_lanes,
-                         bgw::mtxel_fixed_point(ax, c->csize, c->mtxel_lanes) ? bgw::kZyFixed : 0, xp.get())
+            ? mtxel_f64_bands(c, ax, sa, a0, na, sb, b0, nb2, gmap, s.ng, M, s.ng, xp.get())
             : bgw::mtxel_f32(c->slot_ptr(sa, a0), c->slot_ptr(sb, b0), na, nb2, ax, gmap, s.ng, c->A.p, c->Bs.p, M,
                              s.ng, c->st, 0, 0, c->mtxel_lanes, c->mtxel_zy, xp.get(),
                              static_cast<int *>(c->errflag.p));
@@ -1063,6 +1097,7 @@ bgw_status bgw_create(bgw_ctx *out, const int fft[3], int nk, const double *kcry
     c->st = static_cast<cudaStream_t>(stream);
     c->device = dev;
     c->csize = (prec == BGW_FP64) ? 16 : 8;
+    c->fixed = bgw::grid_is_fixed(c->box, c->csize);
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         c->sm_count < 1)
         c->sm_count = 1;

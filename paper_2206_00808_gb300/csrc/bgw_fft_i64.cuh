@@ -289,4 +289,30 @@ __device__ __forceinline__ void fft_line_fix(cpx<double> (&a)[N]) {
     }
 }
 
+// ------------------------------------------------------- integer grids --
+// Real-space grids of the FP64 contexts whose y-z planes are square and at
+// most 40 wide are kept as integers of one scale per (band, x-plane), both
+// spin components together: {re hi, re lo, im hi, im lo} with
+// u = (hi 2^32 + lo) 2^scale, |u| 2^-scale <= 2^fix_grid_top(N).  16 bytes a
+// value, as in FP64; the largest component of a plane keeps 60 bits.
+constexpr int kFixBad = 1 << 24;      // scale of a plane with an infinity or a NaN
+// Pair densities of two such planes stay below 2^fix_top(N).
+__host__ __device__ constexpr int fix_grid_top(int n) { return fix_top(n) >= 58 ? 60 : 59; }
+
+__device__ __forceinline__ int4 fix_pack(long long x, long long y) {
+    fix_parts p = fix_split(x), q = fix_split(y);
+    // -2^31 has no negative: one unit aside instead
+    if (p.l == (int)0x80000000) p.l = -0x7fffffff;
+    if (q.l == (int)0x80000000) q.l = -0x7fffffff;
+    return make_int4(p.h, p.l, q.h, q.l);
+}
+__device__ __forceinline__ long long fix_unpack(int h, int l) { return ((long long)h << 32) + l; }
+
+// |hi word| bits of a value, for the OR over many: all |v| < 2^(64 - clz(OR)).
+__device__ __forceinline__ int fix_mag(i64c v) {
+    const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
+    return (x ^ (x >> 31)) | (y ^ (y >> 31));
+}
+__device__ __forceinline__ long long fix_shift_right(long long v, int r) { return (v + (1LL << (r - 1))) >> r; }
+
 }  // namespace bgw

@@ -10,8 +10,14 @@ cudaError_t mtxel_tables_init_f64();
 cudaError_t bounds_take_mtxel_f64(unsigned *word);
 
 cudaError_t grid_tables_init_f64() {
-    const cudaError_t e = f64::upload_tables();
-    return e == cudaSuccess ? mtxel_tables_init_f64() : e;
+    cudaError_t e = f64::upload_tables();
+    if (e == cudaSuccess) e = mtxel_tables_init_f64();
+    if (e == cudaSuccess) e = grid_fix_tables_init();
+    return e == cudaSuccess ? zy_fix_tables_init() : e;
+}
+cudaError_t wfn_xpass_f64(const double *coeff, int ngw, int B, const int *cube_map, const Axes &a, void *S,
+                          cudaStream_t st) {
+    return f64::wfn_xpass(reinterpret_cast<const double2 *>(coeff), ngw, B, cube_map, a, static_cast<f64::C *>(S), st);
 }
 cudaError_t wfn_to_grid_f64(const double *coeff, int ngw, int B, const int *cube_map,
                             const Axes &a, void *S, void *R, void *U, cudaStream_t st, int path) {

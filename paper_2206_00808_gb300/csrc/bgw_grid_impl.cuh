@@ -1197,6 +1197,14 @@ static cudaError_t launch_fused_batch(const K1Batch &jb, int n, size_t smem, cud
     return cudaGetLastError();
 }
 
+static cudaError_t wfn_xpass(const double2 *cf, int ngw, long nb, const int *cube_map, const Axes &a, C *Sp,
+                             cudaStream_t st) {
+    const long lines = nb * a.w[1] * a.w[2];
+    BGW_FOR_EACH_LEN(a.n[0], (k1_xpass<N><<<blocks_for(lines), kLineThreads, 0, st>>>(
+                                 cf, ngw, nb, cube_map, a.w[0], a.w[1], a.w[2], a.s[0], Sp)));
+    return cudaGetLastError();
+}
+
 static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *cube_map,
                                const Axes &a, void *S, void *R, void *U, cudaStream_t st, int path) {
     const long nb = B;
@@ -1278,11 +1286,8 @@ static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *c
         });
         return cudaGetLastError();
     }
-    {
-        const long lines = nb * a.w[1] * a.w[2];
-        BGW_FOR_EACH_LEN(a.n[0], (k1_xpass<N><<<blocks_for(lines), kLineThreads, 0, st>>>(
-                                     cf, ngw, nb, cube_map, a.w[0], a.w[1], a.w[2], a.s[0], Sp)));
-    }
+    const cudaError_t ex = wfn_xpass(cf, ngw, nb, cube_map, a, Sp, st);
+    if (ex != cudaSuccess) return ex;
 #if BGW_F32
     if (use_plane_kernels(a)) {
         const int n = a.n[1];
@@ -1516,7 +1521,7 @@ static cudaError_t stream_maps(const C *uv, int nvb, const C *uc, int nc, const 
 static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const Axes &a,
                                const int *gmap, int ng, C *Ap, C *Bp, C *Mp, long ldm,
                                cudaStream_t st, int tv_req, int tc_req, int lanes, int zy,
-                               const XPassHook *hook, int *err, int drop) {
+                               const XPassHook *hook, int *err, int drop, const int *sv, const int *sc) {
     const long P = (long)nv * nc;
     if (oct_len(a) && (lanes == 8 || (lanes == 0 && use_coop(a) && use_oct(a)))) {
         // eight lanes per line: fused z+y, then the x pass
@@ -1617,10 +1622,10 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
     }
 #endif
 #if !BGW_F32
-    if (zy == kZyFixed) {
-        const cudaError_t e = mtxel_zy_fix(uv, uc, nv, nc, a, Ap, Bp, st);
+    if (sv) {
+        const cudaError_t e = mtxel_zy_fix(uv, sv, uc, sc, nv, nc, a, Bp, st);
         if (e != cudaSuccess) return e;
-        XMark xm(hook, 3);
+        XMark xm(hook, 1);
         return xpass(Bp, P, a, gmap, ng, Mp, ldm, st);
     }
 #endif
@@ -1699,16 +1704,17 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
 static cudaError_t mtxel(const void *Uv, const void *Uc, int nv, int nc, const Axes &a,
                          const int *gmap, int ng, void *A, void *Bs, void *M, long ldm,
                          cudaStream_t st, int tv_req, int tc_req, int lanes, int zy, const XPassHook *hook,
-                         int *err, int drop) {
+                         int *err, int drop, const int *sv = nullptr, const int *sc = nullptr) {
     if ((long)nv * nc == 0) return cudaSuccess;
     const C *uv = static_cast<const C *>(Uv), *uc = static_cast<const C *>(Uc);
     C *Ap = static_cast<C *>(A), *Bp = static_cast<C *>(Bs), *Mp = static_cast<C *>(M);
     const long vol = (long)a.n[0] * a.n[1] * a.n[2];
-    const int VB = mtxel_v_batch(nv, nc, a, sizeof(C), sizeof(T) == 8 && zy == kZyFixed);
+    const int VB = mtxel_v_batch(nv, nc, a, sizeof(C), sv != nullptr);
     for (int vb0 = 0; vb0 < nv; vb0 += VB) {
         const int nvb = nv - vb0 < VB ? nv - vb0 : VB;
         cudaError_t e = mtxel_batch(uv + (long)vb0 * 2 * vol, uc, nvb, nc, a, gmap, ng, Ap, Bp,
-                                    Mp + (long)vb0 * nc * ldm, ldm, st, tv_req, tc_req, lanes, zy, hook, err, drop);
+                                    Mp + (long)vb0 * nc * ldm, ldm, st, tv_req, tc_req, lanes, zy, hook, err, drop,
+                                    sv ? sv + (long)vb0 * a.n[0] : nullptr, sc);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

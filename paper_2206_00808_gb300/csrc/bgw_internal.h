@@ -62,8 +62,8 @@ cudaError_t wfn_to_grid_batch_f32(const K1Job *jobs, int n, int B, cudaStream_t 
 // N = 32, 40, 48 or 64 (automatic choice uses them for 48 and 64 only).
 // Pairs are processed in batches of mtxel_v_batch(...) valence bands x nc, so
 // A and Bs need room for that many pairs only.
-// zy (FP64): kZyFixed takes the fixed-point z + y kernel (the caller checked
-// mtxel_fixed_point and sized A by mtxel_a_bytes), else the FP64 passes.
+// sv, sc (FP64): the grids are integer grids with these scales, taken by the
+// fixed-point z + y kernel (A unused); null: FP64 grids, the single passes.
 // zy (FP32): 0 automatic (the streamed z + y kernel where it applies, unless a
 // pair tile tv x tc is given), 1 the plane kernel with the pair tile tv x tc,
 // 2 streamed where it applies.
@@ -77,11 +77,10 @@ struct XPassHook {
     void (*fn)(void *ctx, int begin, int kernels);
     void *ctx;
 };
-constexpr int kZyFixed = 3;
 cudaError_t mtxel_f64(const void *Uv, const void *Uc, int nv, int nc, const Axes &a,
                       const int *gmap, int ng, void *A, void *Bs, void *M, long ldm,
-                      cudaStream_t st, int tv = 0, int tc = 0, int lanes = 0, int zy = 0,
-                      const XPassHook *hook = nullptr, int *err = nullptr, int drop = 0);
+                      cudaStream_t st, int lanes = 0, const XPassHook *hook = nullptr, const int *sv = nullptr,
+                      const int *sc = nullptr);
 cudaError_t mtxel_f32(const void *Uv, const void *Uc, int nv, int nc, const Axes &a,
                       const int *gmap, int ng, void *A, void *Bs, void *M, long ldm,
                       cudaStream_t st, int tv = 0, int tc = 0, int lanes = 0, int zy = 0,
@@ -116,22 +115,16 @@ inline bool wfn_uses_r(const Axes &a, size_t csize) {
     return !fp32_square;
 }
 
-// Whether the FP64 matrix elements of a context take the fixed-point z + y
-// kernel (bgw_zy_fix.cu): square y-z planes whose lines fit one thread, unless
-// the eight-lane kernels are asked for.  (bgw_mtxel_spinor_noalloc keeps the
-// FP64 pair density: its grids come from the caller, and one scale per plane
-// is as exact as FP64 only for grids that carry the rounding of a transform.)
-inline bool mtxel_fixed_point(const Axes &a, size_t csize, int lanes) {
-    const bool cubic = a.n[0] == a.n[1] && a.n[1] == a.n[2];
-    return csize == 16 && a.n[1] == a.n[2] && a.n[1] <= 40 && !(lanes == 8 && cubic && (a.n[0] == 32 || a.n[0] == 40));
-}
-// Bands of each side that kernel holds as integers at a time: up to 1 GiB in all.
-inline void fix_band_caps(const Axes &a, int nv, int nc, int *vcap, int *ccap) {
-    const size_t band = (size_t)a.n[0] * (2 * 16 * (size_t)a.n[1] * a.n[2] + sizeof(int));
-    const size_t half = ((size_t)1 << 29) / band;
-    const int cap = half < 1 ? 1 : half > (1u << 20) ? 1 << 20 : (int)half;
-    *vcap = nv < cap ? nv : cap;
-    *ccap = nc < cap ? nc : cap;
+// Whether a context's real-space grids are integer grids (bgw_fft_i64.cuh):
+// FP64 with square y-z planes whose lines fit one thread.  Their matrix
+// elements take the fixed-point z + y kernel (bgw_zy_fix.cu), or, on request
+// for the eight-lane kernels, FP64 copies of the bands in scratch A.
+// (bgw_mtxel_spinor_noalloc has FP64 grids from its caller and keeps the FP64
+// pair density: one scale per plane is as exact as FP64 only for grids that
+// carry the rounding of a transform.)
+inline bool grid_is_fixed(const int *n, size_t csize) { return csize == 16 && n[1] == n[2] && n[1] <= 40; }
+inline bool mtxel_eight_lanes(const int *n, int lanes) {
+    return lanes == 8 && n[0] == n[1] && n[1] == n[2] && (n[0] == 32 || n[0] == 40);
 }
 
 // Valence bands per batch of the matrix-element kernels: their scratch
@@ -151,22 +144,28 @@ inline int mtxel_v_batch(int nv, int nc, const Axes &a, size_t csize, bool fixed
     if (vb >= group) vb -= vb % group;
     return (int)vb;
 }
-// Bytes of scratch A for one such batch: the z-pass output of its pairs, or the
-// bands of the fixed-point kernel.
+// Bytes of scratch A for one such batch: the z-pass output of its pairs.
 inline size_t mtxel_a_bytes(int nv, int nc, const Axes &a, size_t csize, bool fixed) {
-    const int vb = mtxel_v_batch(nv, nc, a, csize, fixed);
-    if (fixed) {
-        int vcap, ccap;
-        fix_band_caps(a, vb, nc, &vcap, &ccap);
-        return (size_t)(vcap + ccap) * a.n[0] * (2 * 16 * (size_t)a.n[1] * a.n[2] + sizeof(int));
-    }
-    return mtxel_uses_a(a) ? (size_t)vb * nc * a.n[0] * a.n[1] * a.w[2] * csize : 0;
+    if (fixed || !mtxel_uses_a(a)) return 0;
+    return (size_t)mtxel_v_batch(nv, nc, a, csize, fixed) * nc * a.n[0] * a.n[1] * a.w[2] * csize;
 }
-// z + y passes of nv x nc pairs into Bs (see mtxel_f64), FP64 through 64-bit
-// fixed point; ws: mtxel_a_bytes of scratch.
+
+// ---- integer grids (bgw_grid_fix.cu, bgw_zy_fix.cu) -----------------------
+cudaError_t grid_fix_tables_init();
 cudaError_t zy_fix_tables_init();
-cudaError_t mtxel_zy_fix(const void *Uv, const void *Uc, int nv, int nc, const Axes &a, void *ws, void *Bs,
-                         cudaStream_t st);
+// x pass of wfn_to_grid_f64 (B band components) into S.
+cudaError_t wfn_xpass_f64(const double *coeff, int ngw, int B, const int *cube_map, const Axes &a, void *S,
+                          cudaStream_t st);
+// wfn_to_grid for nb bands into an integer grid: U [nb][2][N^3] of 16 bytes,
+// scale [nb][n0].
+cudaError_t wfn_to_fix(const double *coeff, int ngw, int nb, const int *cube_map, const Axes &a, void *S, void *U,
+                       int *scale, cudaStream_t st);
+// FP64 grid to integer grid in place, and an integer grid to an FP64 one.
+cudaError_t grid_to_fix(void *U, int nb, const Axes &a, int *scale, cudaStream_t st);
+cudaError_t fix_to_grid(const void *F, const int *scale, int nb, const Axes &a, void *U, cudaStream_t st);
+// z + y passes of nv x nc pairs of two integer grids into Bs (see mtxel_f64).
+cudaError_t mtxel_zy_fix(const void *Fv, const int *Sv, const void *Fc, const int *Sc, int nv, int nc, const Axes &a,
+                         void *Bs, cudaStream_t st);
 
 // Candidate pair tiles (tv, tc) of the plane-fused FP32 kernel for this shape,
 // best first by the staging heuristic; returns how many were written.

@@ -1,9 +1,8 @@
 // Pair density + z and y passes of the FP64 matrix elements in 64-bit fixed
 // point, for boxes with N2 = N3 <= 40 (Eq. matrix_el of arXiv:2206.00808).
 //
-// k2_fix_planes writes every band's x-planes as integers of one scale per
-// (band, x-plane), split for the multiplier: {re hi, re lo, im hi, im lo}.
-// k2_zy_fix then takes one x-plane and a tile of TV x TC pairs per CTA:
+// k2_zy_fix reads integer grids (bgw_fft_i64.cuh) and takes one x-plane and a
+// tile of TV x TC pairs per CTA:
 //   1. rho = sum_alpha conj(u_v) u_c at every point of the plane, a thread per
 //      point with the tile's TV + TC values in registers (24 multiply-adds and
 //      two joins a pair and point), into shared memory [pair][y][z];
@@ -24,51 +23,7 @@
 namespace bgw {
 namespace {
 
-constexpr int kFixBad = 1 << 24;      // scale of a plane with an infinity or a NaN
-constexpr int kConvThreads = 256;
 constexpr int kWinF = 8;              // kept outputs within +-kWinF of 0 let the compiler drop butterflies
-
-// |u| of a plane below 2^kTopU: rho stays below fix_top(N).
-__host__ __device__ constexpr int zy_top_u(int n) { return fix_top(n) >= 58 ? 60 : 59; }
-
-// One CTA per (x-plane, band): both spin components.
-template <int N>
-__global__ void __launch_bounds__(kConvThreads)
-k2_fix_planes(const double2 *__restrict__ U, int4 *__restrict__ F, int *__restrict__ scale) {
-    constexpr int NN = N * N, IT = (2 * NN + kConvThreads - 1) / kConvThreads;
-    const int x = blockIdx.x, n0 = gridDim.x;
-    const long b = blockIdx.y;
-    __shared__ int smax;
-    if (threadIdx.x == 0) smax = 0;
-    double2 v[IT];
-    int m = 0;
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-        const int t = i * kConvThreads + threadIdx.x;
-        v[i] = make_double2(0.0, 0.0);
-        if (t < 2 * NN) v[i] = U[((2 * b + t / NN) * n0 + x) * NN + t % NN];
-        m = max(m, max(__double2hiint(v[i].x) & 0x7fffffff, __double2hiint(v[i].y) & 0x7fffffff));
-    }
-    __syncthreads();
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(&smax, m);
-    __syncthreads();
-    const int E = smax >> 20;
-    constexpr int TOP = zy_top_u(N);
-    if (threadIdx.x == 0) scale[b * n0 + x] = E == 0x7ff ? kFixBad : E - 1022 - TOP;
-    int4 *o = F + (b * n0 + x) * 2L * NN;
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-        const int t = i * kConvThreads + threadIdx.x;
-        if (t < 2 * NN) {
-            fix_parts p = fix_split(fix_in<TOP>(v[i].x, E)), q = fix_split(fix_in<TOP>(v[i].y, E));
-            // -2^31 has no negative: one unit of 2^-60 aside instead
-            if (p.l == (int)0x80000000) p.l = -0x7fffffff;
-            if (q.l == (int)0x80000000) q.l = -0x7fffffff;
-            o[t] = make_int4(p.h, p.l, q.h, q.l);
-        }
-    }
-}
 
 template <int N>
 struct ZyTile {
@@ -97,20 +52,21 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
     // 1. pair densities (a tile's missing bands repeat its last one)
     const int4 *pv[TV], *pc[TC];
 #pragma unroll
-    for (int v = 0; v < TV; ++v) pv[v] = Fv + ((long)(v0 + min(v, tv - 1)) * n0 + x) * 2 * NN;
+    for (int v = 0; v < TV; ++v) pv[v] = Fv + (2L * (v0 + min(v, tv - 1)) * n0 + x) * NN;
 #pragma unroll
-    for (int c = 0; c < TC; ++c) pc[c] = Fc + ((long)(c0 + min(c, tc - 1)) * n0 + x) * 2 * NN;
+    for (int c = 0; c < TC; ++c) pc[c] = Fc + (2L * (c0 + min(c, tc - 1)) * n0 + x) * NN;
+    const long spin = (long)n0 * NN;
     for (int t = threadIdx.x; t < NN; t += THREADS) {
         int4 c[TC][2];
 #pragma unroll
         for (int i = 0; i < TC; ++i) {
             c[i][0] = __ldg(pc[i] + t);
-            c[i][1] = __ldg(pc[i] + NN + t);
+            c[i][1] = __ldg(pc[i] + spin + t);
         }
         i64c *r = R + (t / N) * RS + t % N;
 #pragma unroll
         for (int v = 0; v < TV; ++v) {
-            const int4 a = __ldg(pv[v] + t), b = __ldg(pv[v] + NN + t);
+            const int4 a = __ldg(pv[v] + t), b = __ldg(pv[v] + spin + t);
             const int nah = -a.z, nal = -a.w, nbh = -b.z, nbl = -b.w;      // minus the imaginary parts
 #pragma unroll
             for (int i = 0; i < TC; ++i) {
@@ -144,8 +100,7 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
                 const int j = f + ns2 >= N ? f + ns2 - N : f + ns2;
                 if (j < w2) {
                     row[j] = a[f];
-                    const int hx = (int)(a[f].x >> 32), hy = (int)(a[f].y >> 32);
-                    big |= (hx ^ (hx >> 31)) | (hy ^ (hy >> 31));
+                    big |= fix_mag(a[f]);
                 }
             }
             atomicMax(&pbits[pr], 64 - __clz(big));      // every kept |value| <= 2^bits
@@ -163,9 +118,8 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
 #pragma unroll
         for (int y = 0; y < N; ++y) a[y] = col[y * RS];
         if (r > 0) {
-            const long long half = 1LL << (r - 1);
 #pragma unroll
-            for (int y = 0; y < N; ++y) a[y] = i64c{(a[y].x + half) >> r, (a[y].y + half) >> r};
+            for (int y = 0; y < N; ++y) a[y] = i64c{fix_shift_right(a[y].x, r), fix_shift_right(a[y].y, r)};
         }
         FixFft<-1, N, N>::run(a);
         const int ev = Sv[(long)(v0 + v) * n0 + x], ec = Sc[(long)(c0 + c) * n0 + x];
@@ -196,31 +150,15 @@ bool in_window(const Axes &a, int ax) {
 }
 
 template <int N>
-cudaError_t zy_fix_n(const double2 *uv, const double2 *uc, int nv, int nc, const Axes &a, void *ws, double2 *Bs,
-                     cudaStream_t st) {
+cudaError_t zy_fix_n(const int4 *fv, const int *sv, const int4 *fc, const int *sc, int nv, int nc, const Axes &a,
+                     double2 *Bs, cudaStream_t st) {
     using Tile = ZyTile<N>;
-    const int n0 = a.n[0];
-    const long plane_vals = (long)n0 * 2 * N * N;
-    int vcap, ccap;
-    fix_band_caps(a, nv, nc, &vcap, &ccap);
-    int4 *Fv = static_cast<int4 *>(ws), *Fc = Fv + (long)vcap * plane_vals;
-    int *Sv = reinterpret_cast<int *>(Fc + (long)ccap * plane_vals), *Sc = Sv + (long)vcap * n0;
     auto kern = k2_zy_fix<N, false>;
     if (in_window(a, 1) && in_window(a, 2)) kern = k2_zy_fix<N, (N > 2 * kWinF + 1)>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile::SMEM);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile::SMEM);
     if (e != cudaSuccess) return e;
-    for (int v = 0; v < nv; v += vcap) {
-        const int kv = nv - v < vcap ? nv - v : vcap;
-        k2_fix_planes<N><<<dim3(n0, kv), kConvThreads, 0, st>>>(uv + v * plane_vals, Fv, Sv);
-        for (int c = 0; c < nc; c += ccap) {
-            const int kc = nc - c < ccap ? nc - c : ccap;
-            k2_fix_planes<N><<<dim3(n0, kc), kConvThreads, 0, st>>>(uc + c * plane_vals, Fc, Sc);
-            const dim3 grid(n0, (kv + Tile::TV - 1) / Tile::TV, (kc + Tile::TC - 1) / Tile::TC);
-            kern<<<grid, Tile::THREADS, Tile::SMEM, st>>>(
-                Fv, Sv, Fc, Sc, kv, kc, nc, a.w[1], a.w[2], a.s[1], a.s[2],
-                Bs + ((long)v * nc + c) * n0 * a.w[1] * (long)a.w[2]);
-        }
-    }
+    const dim3 grid(a.n[0], (nv + Tile::TV - 1) / Tile::TV, (nc + Tile::TC - 1) / Tile::TC);
+    kern<<<grid, Tile::THREADS, Tile::SMEM, st>>>(fv, sv, fc, sc, nv, nc, nc, a.w[1], a.w[2], a.s[1], a.s[2], Bs);
     return cudaGetLastError();
 }
 
@@ -234,20 +172,20 @@ cudaError_t zy_fix_tables_init() {
     return e == cudaSuccess ? cudaMemcpyToSymbol(c_consq, cq, sizeof cq) : e;
 }
 
-cudaError_t mtxel_zy_fix(const void *Uv, const void *Uc, int nv, int nc, const Axes &a, void *ws, void *Bs,
-                         cudaStream_t st) {
-    const double2 *uv = static_cast<const double2 *>(Uv), *uc = static_cast<const double2 *>(Uc);
+cudaError_t mtxel_zy_fix(const void *Fv, const int *Sv, const void *Fc, const int *Sc, int nv, int nc, const Axes &a,
+                         void *Bs, cudaStream_t st) {
+    const int4 *fv = static_cast<const int4 *>(Fv), *fc = static_cast<const int4 *>(Fc);
     double2 *b = static_cast<double2 *>(Bs);
     switch (a.n[1]) {
-        case 16: return zy_fix_n<16>(uv, uc, nv, nc, a, ws, b, st);
-        case 18: return zy_fix_n<18>(uv, uc, nv, nc, a, ws, b, st);
-        case 20: return zy_fix_n<20>(uv, uc, nv, nc, a, ws, b, st);
-        case 24: return zy_fix_n<24>(uv, uc, nv, nc, a, ws, b, st);
-        case 27: return zy_fix_n<27>(uv, uc, nv, nc, a, ws, b, st);
-        case 30: return zy_fix_n<30>(uv, uc, nv, nc, a, ws, b, st);
-        case 32: return zy_fix_n<32>(uv, uc, nv, nc, a, ws, b, st);
-        case 36: return zy_fix_n<36>(uv, uc, nv, nc, a, ws, b, st);
-        case 40: return zy_fix_n<40>(uv, uc, nv, nc, a, ws, b, st);
+        case 16: return zy_fix_n<16>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 18: return zy_fix_n<18>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 20: return zy_fix_n<20>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 24: return zy_fix_n<24>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 27: return zy_fix_n<27>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 30: return zy_fix_n<30>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 32: return zy_fix_n<32>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 36: return zy_fix_n<36>(fv, Sv, fc, Sc, nv, nc, a, b, st);
+        case 40: return zy_fix_n<40>(fv, Sv, fc, Sc, nv, nc, a, b, st);
         default: return cudaErrorInvalidValue;
     }
 }
