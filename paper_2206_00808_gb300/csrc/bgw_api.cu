@@ -26,6 +26,7 @@
 #include "bgw_internal.h"
 #include "bgw_mixed.h"
 #include "bgw_f64tc.h"
+#include "bgw_dz.h"
 
 namespace {
 
@@ -171,7 +172,7 @@ struct bgw_ctx_s {
     DevBuf errflag;      // device int: non-zero after a bounded device wait gave up
     // scratch of the self-energy and BSE kernel calls (matrix-element blocks,
     // products, per-pair sums, a copy of the interaction's diagonal)
-    DevBuf nx_m1, nx_m2, nx_y, nx_t, nx_s, nx_v;
+    DevBuf nx_m1, nx_m2, nx_y, nx_t, nx_s, nx_v, nx_dz;
     // real-space grid slots: every k resident (nslots == nk), or a
     // least-recently-used cache of nslots grids (streaming)
     int grid_slots_opt = 0;
@@ -964,6 +965,40 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
     xp.finish();
     if (e != cudaSuccess) return c->cuda_fail(e, "matrix-element kernels");
     return BGW_OK;
+}
+
+// C[m][n] = alpha sum_k opA[m][k] wk[k] opB[n][k] with rows of both operands
+// contiguous (row strides sa, sb; C row stride sc): on tensor cores from digit
+// slices (bgw_dz.cu), in pieces of at most 512 MiB of digits per operand.
+// Short sums stay on the FP64 kernel, which rounds every product on its own
+// scale: the slices' 2^-56 of the rows' largest products is below the rounding
+// of an FP64 sum only once that sum has some tens of terms.
+constexpr int kDzMinK = 32;
+cudaError_t row_product(bgw_ctx_s *c, long M, int N, int K, const void *A, long sa, bool conjA, const void *B, long sb,
+                        bool conjB, const double *wk, void *C, long sc, double alpha) {
+    if (K < kDzMinK || K > bgw::kDzMaxK)
+        return bgw::zgemm_f64((int)M, N, K, A, sa, 1, conjA, B, 1, sb, conjB, wk, C, sc, 1, alpha, 0.0, false, c->st);
+    const size_t cap = (size_t)512 << 20;
+    auto piece = [&](long rows, bool b) {
+        const size_t one = bgw::dz_planes_bytes(128, K, 1, b) / 128 + 1;
+        return std::min(rows, std::max(128L, (long)(cap / one) / 128 * 128));
+    };
+    const int mp = (int)piece(M, false), np = (int)piece(N, true);
+    const size_t abytes = bgw::dz_planes_bytes(mp, K, 1, false);
+    cudaError_t e = c->nx_dz.ensure(abytes + bgw::dz_planes_bytes(np, K, 1, true), c->st);
+    char *ws = static_cast<char *>(c->nx_dz.p);
+    const double2 *a = static_cast<const double2 *>(A), *b = static_cast<const double2 *>(B);
+    for (int n0 = 0; n0 < N && e == cudaSuccess; n0 += np)
+        for (long m0 = 0; m0 < M && e == cudaSuccess; m0 += mp) {
+            const int m = (int)std::min<long>(mp, M - m0), n = std::min(np, N - n0);
+            const bgw::DzPlanes pl[2] = {bgw::dz_planes(ws, m, K, 1, false), bgw::dz_planes(ws + abytes, n, K, 1, true)};
+            const bgw::DzOperand op[2] = {{a + m0 * sa, 0, sa, 1, conjA, wk}, {b + (long)n0 * sb, 0, sb, 1, conjB, nullptr}};
+            e = bgw::dz_split(op, pl, 2, K, c->st);
+            const bgw::DzOut out = {static_cast<double2 *>(C) + m0 * sc + n0, 0, sc, 1, 0, 0, alpha, 0.0, false};
+            if (e == cudaSuccess)
+                e = bgw::dz_gemm(pl[0], pl[1], out, c->sm_count, c->st, static_cast<int *>(c->errflag.p));
+        }
+    return e;
 }
 
 // Grid index j of k - q: the k-point whose k + q lands on kcrys[ik].
@@ -1860,7 +1895,7 @@ void bgw_destroy(bgw_ctx c) {
         }
         DevBuf *bufs[] = {&c->grids, &c->energy, &c->stage, &c->S,  &c->R,        &c->A,
                           &c->Bs,    &c->M,      &c->W,     &c->mixed_ws, &c->freq_dev, &c->out_stage, &c->gmap_tmp,
-                          &c->errflag, &c->nx_m1, &c->nx_m2, &c->nx_y, &c->nx_t, &c->nx_s, &c->nx_v};
+                          &c->errflag, &c->nx_m1, &c->nx_m2, &c->nx_y, &c->nx_t, &c->nx_s, &c->nx_v, &c->nx_dz};
         for (DevBuf *b : bufs) b->release();
     }
     delete c;
@@ -1940,8 +1975,7 @@ bgw_status bgw_sigma_cohsex(bgw_ctx c, const bgw_q *q, int ik, int n0, int nn, c
     e = cudaMemcpyAsync(c->nx_v.p, vq, sizeof(double) * s.ng, cudaMemcpyHostToDevice, c->st);
     // Y[p][G] = sum_G' W[G][G'] M[p][G']
     if (e == cudaSuccess)
-        e = bgw::zgemm_f64((int)P, s.ng, s.ng, c->nx_m1.p, s.ng, 1, false, W_dev, 1, s.ng, false, nullptr, c->nx_y.p,
-                           s.ng, 1, 1.0, 0.0, false, c->st);
+        e = row_product(c, P, s.ng, s.ng, c->nx_m1.p, s.ng, false, W_dev, s.ng, false, nullptr, c->nx_y.p, s.ng, 1.0);
     if (e == cudaSuccess)
         e = bgw::rowdot_f64(c->nx_m1.p, c->nx_y.p, static_cast<const double *>(c->nx_v.p), P, s.ng, sw, tv, c->st);
     if (e == cudaSuccess) e = bgw::band_sum_f64(sw, c->nv, nn, out, c->st);              // occupied n''
@@ -1950,8 +1984,14 @@ bgw_status bgw_sigma_cohsex(bgw_ctx c, const bgw_q *q, int ik, int n0, int nn, c
     std::vector<double> h(3 * (size_t)nn);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h.data(), out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->st);
+    int flag = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     if (e != cudaSuccess) return c->cuda_fail(e, "sigma_cohsex: kernels");
+    if (flag && flag != bgw::F64TC_ERR_SIGN) {        // a bounded wait of the product gave up: sx, coh unchanged
+        cudaMemsetAsync(c->errflag.p, 0, sizeof(int), c->st);
+        return c->fail(BGW_E_TIMEOUT, "sigma_cohsex: a device-side wait gave up (code %d)", flag);
+    }
     const double scale = 1.0 / c->nk;
     for (int n = 0; n < nn; ++n) {
         sx[n] += -scale * h[n];
@@ -1998,8 +2038,8 @@ bgw_status bgw_bse_kernel(bgw_ctx c, int ik, int jk, const bgw_q *q0, const doub
         e = cudaMemcpyAsync(c->nx_v.p, v0_coul, sizeof(double) * s.ng, cudaMemcpyHostToDevice, c->st);
         // KX[I][J] = (1/N_k) sum_G v(G) M_I(k_i, G) conj(M_J(k_j, G))
         if (e == cudaSuccess)
-            e = bgw::zgemm_f64((int)P, (int)P, s.ng, c->nx_m1.p, s.ng, 1, false, c->nx_m2.p, 1, s.ng, true,
-                               static_cast<const double *>(c->nx_v.p), KX_dev, P, 1, scale, 0.0, false, c->st);
+            e = row_product(c, P, (int)P, s.ng, c->nx_m1.p, s.ng, false, c->nx_m2.p, s.ng, true,
+                            static_cast<const double *>(c->nx_v.p), KX_dev, P, scale);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);   // the host copy of v(G) has been read
         if (e != cudaSuccess) return c->cuda_fail(e, "bse_kernel: exchange");
     }
@@ -2022,12 +2062,11 @@ bgw_status bgw_bse_kernel(bgw_ctx c, int ik, int jk, const bgw_q *q0, const doub
         if (st != BGW_OK) return st;
         const int nv2 = nv * nv, nc2 = nc * nc;
         // Y[(v v')][G] = sum_G' W[G][G'] M_vv'(G')
-        e = bgw::zgemm_f64(nv2, s.ng, s.ng, c->nx_m2.p, s.ng, 1, false, W_dev, 1, s.ng, false, nullptr, c->nx_y.p,
-                           s.ng, 1, 1.0, 0.0, false, c->st);
+        e = row_product(c, nv2, s.ng, s.ng, c->nx_m2.p, s.ng, false, W_dev, s.ng, false, nullptr, c->nx_y.p, s.ng, 1.0);
         // T[(c c')][(v v')] = -(1/N_k) sum_G conj(M_cc'(G)) Y[(v v')][G]
         if (e == cudaSuccess)
-            e = bgw::zgemm_f64(nc2, nv2, s.ng, c->nx_m1.p, s.ng, 1, true, c->nx_y.p, 1, s.ng, false, nullptr,
-                               c->nx_t.p, nv2, 1, -scale, 0.0, false, c->st);
+            e = row_product(c, nc2, nv2, s.ng, c->nx_m1.p, s.ng, true, c->nx_y.p, s.ng, false, nullptr, c->nx_t.p, nv2,
+                            -scale);
         if (e == cudaSuccess) e = bgw::bse_permute_f64(c->nx_t.p, nv, nc, KD_dev, c->st);
         if (e != cudaSuccess) return c->cuda_fail(e, "bse_kernel: direct");
     }

@@ -25,13 +25,18 @@ namespace {
 
 constexpr int kWinF = 8;              // kept outputs within +-kWinF of 0 let the compiler drop butterflies
 
+// Pairs per CTA, one z line per thread: as many as shared memory and the
+// registers of a line leave room for.  Measured per shape: 24^3 (1600 pairs)
+// 2 x 5 pairs at 128 registers 225 us, 2 x 4 at 168 240, 1 x 5 251, 4 x 4 253,
+// 2 x 2 256; 32^3 (1782 pairs) 2 x 4 one CTA per SM 626 us, 2 x 3 656, 2 x 2
+// 677, 1 x 4 730.
 template <int N>
 struct ZyTile {
     static constexpr int TV = 2;
-    static constexpr int TC = N <= 27 ? 4 : N <= 32 ? 3 : 2;
+    static constexpr int TC = N == 24 ? 5 : N <= 27 || N == 32 ? 4 : N == 30 ? 3 : 2;
     static constexpr int RS = N | 1;                                   // odd row: conflict-free 16-byte rows
-    static constexpr int THREADS = (TV * TC * N + 31) / 32 * 32;       // one z line per thread
-    static constexpr int MINB = N == 16 ? 4 : N <= 20 ? 3 : 2;
+    static constexpr int THREADS = (TV * TC * N + 31) / 32 * 32;
+    static constexpr int MINB = N == 16 ? 4 : N <= 20 ? 3 : N == 32 ? 1 : 2;
     static constexpr size_t SMEM = (size_t)TV * TC * N * RS * 16;
 };
 
