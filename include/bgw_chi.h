@@ -286,8 +286,8 @@ BGW_API bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, int
  *   reciprocal vector G0 (Rk = k' + G0), the caller adds G0 to gvec_out
  *   before uploading at k'.  gvec_out is written before the call returns;
  *   c_out when the stream reaches the call.  Uses a stream-ordered device
- *   allocation of 12 ngw bytes (the Miller list; the phases are formed on the
- *   device).  BGW_E_ARG on bad arguments, as for
+ *   allocation of 76 ngw bytes (the Miller list and, per plane wave, U with its
+ *   phase).  BGW_E_ARG on bad arguments, as for
  *   bgw_symmetry_su2, or aliasing; errors via bgw_last_error(NULL).
  */
 BGW_API bgw_status bgw_symmetry_su2(const double *avec, const int *rot_lat, double *U, double *axis_angle);

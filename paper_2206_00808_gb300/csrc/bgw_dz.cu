@@ -63,7 +63,8 @@ struct SplitOp {
     __nv_bfloat16 *x;
     int *scale;
     int rows, rows_pad, b;
-    long tiles;        // 128-row tiles of the whole operand
+    int batch0;        // first matrix of the planes written
+    long tiles;        // 128-row tiles of the planes
     unsigned first;    // first block of this operand
 };
 struct SplitArgs {
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(kSpThreads) k_dz_split(const __grid_constant__
     __syncthreads();
     if (t < kSpRows && r0 + t < o.rows) {
         const int E = smax[t] >> 20;
-        o.scale[(long)b * o.rows + r0 + t] = E == 0x7ff ? kFixBad : E - 1022 - kTopD + 8 * (kSl - 1);
+        o.scale[(long)(o.batch0 + b) * o.rows + r0 + t] = E == 0x7ff ? kFixBad : E - 1022 - kTopD + 8 * (kSl - 1);
     }
     const int rr = t / 8, seg = t % 8;                // this thread's row and pair of complex values
     const int E = smax[rr] >> 20;
@@ -175,13 +176,13 @@ __global__ void __launch_bounds__(kSpThreads) k_dz_split(const __grid_constant__
             n[2 * i + 1] = fix_in<kTopD>(v[i].y, E);
         }
         if (o.b) {
-            const long row = (long)b * o.rows_pad + 2 * (r0 + rr);
+            const long row = (long)(o.batch0 + b) * o.rows_pad + 2 * (r0 + rr);
             __nv_bfloat16 *x = o.x + ((row / kM * a.kblocks + kb) * kM + row % kM) * kKB + 4 * seg;
             const long long p[4] = {n[0], -n[1], n[2], -n[3]}, q[4] = {n[1], n[0], n[3], n[2]};
             dz_store(x, plane, p);
             dz_store(x + kKB, plane, q);
         } else {
-            const long row = (long)b * o.rows_pad + r0 + rr;
+            const long row = (long)(o.batch0 + b) * o.rows_pad + r0 + rr;
             dz_store(o.x + ((row / kM * a.kblocks + kb) * kM + row % kM) * kKB + 4 * seg, plane, n);
         }
     }
@@ -229,13 +230,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+enum { kOne, kMinusOne, kReal, kComplex };
 struct GemmArgs {
     CUtensorMap ma, mb;
     const int *ea, *eb;      // scales [batch][M], [batch][N]
     DzOut out;
     int M, N, ta, tb;        // rows, columns, tiles per matrix
     int rpa, rpb;            // padded rows per matrix of each operand
+    int b0a, b0b;            // first matrix of each operand's planes
     int nkb, items;
+    int alpha;               // kOne ...: no FP64 compare per output
 };
 
 __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__ GemmArgs g, int *__restrict__ err) {
@@ -273,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
             bool stop = false;
             for (int item = blockIdx.x; item < g.items && !stop; item += gridDim.x) {
                 const int b = item / per, ti = item % per / g.tb, tj = item % per % g.tb;
-                const int ra = b * g.rpa + ti * kM, rb = b * g.rpb + tj * kN;
+                const int ra = (g.b0a + b) * g.rpa + ti * kM, rb = (g.b0b + b) * g.rpb + tj * kN;
                 for (int kb = 0; kb < g.nkb; ++kb, ++pit) {
                     const int s = (int)(pit % kStg);
                     if (!mbar_wait(smem_u32(&empty_bar[s]), (uint32_t)(((pit / kStg) & 1) ^ 1))) {
@@ -379,21 +383,30 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 uint32_t v[16];
-                float s = 1.0f;
+                int h[16];
+                // orders 0 and 1 (below 2^20 and 2^21 units), 2 and 3 (2^23, 2^24) join in 32 bits
 #pragma unroll
-                for (int o = 0; o < kAcc - 1; ++o) {
+                for (int o = 0; o < 4; o += 2) {
+                    const float s0 = o ? 0x1p16f : 1.0f, s1 = o ? 0x1p24f : 0x1p8f;
                     tmem_ld16(lane_base + (uint32_t)(o * kN), v);
 #pragma unroll
+                    for (int i = 0; i < 16; ++i) h[i] = __float2int_rn(__uint_as_float(v[i]) * s0) * 256;
+                    tmem_ld16(lane_base + (uint32_t)((o + 1) * kN), v);
+#pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const int d = __float2int_rn(__uint_as_float(v[i]) * s);
-                        if (o < kAcc - 2) {
-                            n[i] += (long long)d << (36 - 8 * o);
-                        } else {
-                            n[i] += d >> 4;
-                            f[i] += (float)(d & 15) * 0x1p-40f;
-                        }
+                        const int d = h[i] + __float2int_rn(__uint_as_float(v[i]) * s1);
+                        n[i] += (long long)d << (o ? 12 : 28);
                     }
-                    s *= 256.0f;
+                }
+                tmem_ld16(lane_base + (uint32_t)(4 * kN), v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) n[i] += (long long)__float2int_rn(__uint_as_float(v[i]) * 0x1p32f) << 4;
+                tmem_ld16(lane_base + (uint32_t)(5 * kN), v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int d = __float2int_rn(__uint_as_float(v[i]) * 0x1p40f);
+                    n[i] += d >> 4;
+                    f[i] += (float)(d & 15) * 0x1p-40f;
                 }
                 tmem_ld16(lane_base + (uint32_t)((kAcc - 1) * kN), v);
 #pragma unroll
@@ -409,40 +422,37 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
             const int n0 = (tj * kN + 16 * group) / 2;
             const DzOut &o = g.out;
             if (m < g.M && !(m >= o.skip0 && m < o.skip1)) {
-                const int ea = g.ea[(long)b * g.M + m];
-                double2 *c = o.c + b * o.sb + m * o.sm;
+                const int ea = g.ea[(long)(g.b0a + b) * g.M + m];
+                const int *ebp = g.eb + (long)(g.b0b + b) * g.N;
+                double2 *c = o.c + b * o.sb + m * o.sm + n0 * o.sn;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int nn = n0 + i;
-                    if (nn < g.N && !(nn >= o.skip0 && nn < o.skip1)) {
-                        const int eb = g.eb[(long)b * g.N + nn];
-                        double d[2];
+                    if (nn >= g.N || (nn >= o.skip0 && nn < o.skip1)) continue;
+                    const int eb = ebp[nn];
+                    double2 *p = c + i * o.sn;
+                    double2 old = make_double2(0.0, 0.0);
+                    if (o.accumulate) old = *p;
+                    double d[2];
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int q = 2 * i + h;
-                            long long x = n[q];
-                            // the last sum is a fraction of x's unit: bring x up to make room for it
-                            const int sh = min(max(__clzll(x < 0 ? ~x : x) - 2, 0), 26);
-                            x = (x << sh) + __float2ll_rn(f[q] * __int_as_float((127 + 36 + sh) << 23));
-                            d[h] = fix_out(x, 1086 - 36 - sh + ea + eb);
-                        }
-                        double2 r = make_double2(d[0], d[1]);
-                        if (ea == kFixBad || eb == kFixBad)
-                            r.x = r.y = __longlong_as_double(0x7ff8000000000000ll);
-                        if (o.ai != 0.0)
-                            r = make_double2(o.ar * r.x - o.ai * r.y, o.ar * r.y + o.ai * r.x);
-                        else if (o.ar == -1.0)
-                            r = make_double2(-r.x, -r.y);
-                        else if (o.ar != 1.0)
-                            r = make_double2(o.ar * r.x, o.ar * r.y);
-                        double2 *p = c + nn * o.sn;
-                        if (o.accumulate) {
-                            const double2 old = *p;
-                            r.x += old.x;
-                            r.y += old.y;
-                        }
-                        *p = r;
+                    for (int h = 0; h < 2; ++h) {
+                        const int q = 2 * i + h;
+                        long long x = n[q];
+                        // the last sum is a fraction of x's unit: bring x up to make room for it
+                        const int sh = min(max(__clzll(x < 0 ? ~x : x) - 2, 0), 26);
+                        const long long fr = __float2int_rn(f[q] * 0x1p52f);      // units of 2^-52
+                        x = (x << sh) + (sh >= 16 ? fr << (sh - 16) : fr >> (16 - sh));
+                        if (g.alpha == kMinusOne) x = -x;
+                        d[h] = fix_out(x, 1086 - 36 - sh + ea + eb);
                     }
+                    double2 r = make_double2(d[0], d[1]);
+                    if (ea == kFixBad || eb == kFixBad) r.x = r.y = __longlong_as_double(0x7ff8000000000000ll);
+                    if (g.alpha == kComplex)
+                        r = make_double2(o.ar * r.x - o.ai * r.y, o.ar * r.y + o.ai * r.x);
+                    else if (g.alpha == kReal)
+                        r = make_double2(o.ar * r.x, o.ar * r.y);
+                    if (o.accumulate) r = make_double2(r.x + old.x, r.y + old.y);
+                    *p = r;
                 }
             }
         }
@@ -483,7 +493,8 @@ DzPlanes dz_planes(void *ws, int rows, int K, int batch, bool b) {
     p.rows = rows;
     p.rows_pad = pad_rows(rows, b);
     p.kblocks = (int)(round_up(2L * K, kKB) / kKB);
-    p.batch = batch;
+    p.batch = p.used = batch;
+    p.first = 0;
     p.b = b;
     p.scale = reinterpret_cast<int *>(static_cast<char *>(ws) + plane_bytes(p));
     return p;
@@ -504,8 +515,8 @@ cudaError_t dz_split(const DzOperand *op, const DzPlanes *pl, int n, int K, cuda
     for (int i = 0; i < n; ++i) {
         const DzPlanes &p = pl[i];
         a.o[i] = SplitOp{op[i], static_cast<__nv_bfloat16 *>(p.x), p.scale, p.rows, p.rows_pad, p.b ? 1 : 0,
-                         tile_rows(p) / kM, blocks};
-        blocks += (unsigned)(p.batch * (p.rows_pad / (p.b ? 2 * kSpRows : kSpRows)));
+                         p.first, tile_rows(p) / kM, blocks};
+        blocks += (unsigned)(p.used * (p.rows_pad / (p.b ? 2 * kSpRows : kSpRows)));
     }
     k_dz_split<<<blocks, kSpThreads, 0, st>>>(a);
     return cudaGetLastError();
@@ -527,7 +538,10 @@ cudaError_t dz_gemm(const DzPlanes &A, const DzPlanes &B, const DzOut &out, int 
     g.ta = A.rows_pad / kM;
     g.tb = B.rows_pad / kN;
     g.nkb = A.kblocks;
-    g.items = A.batch * g.ta * g.tb;
+    g.b0a = A.first;
+    g.b0b = B.first;
+    g.items = A.used * g.ta * g.tb;
+    g.alpha = out.ai != 0.0 ? kComplex : out.ar == 1.0 ? kOne : out.ar == -1.0 ? kMinusOne : kReal;
     const int smem = kStg * kStage + 1024;
     e = cudaFuncSetAttribute(k_dz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

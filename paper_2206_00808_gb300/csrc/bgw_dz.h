@@ -21,7 +21,9 @@ struct DzOperand {
 struct DzPlanes {
     void *x;          // BF16 digits
     int *scale;       // exponent of each (batch, row)
-    int rows, rows_pad, kblocks, batch;
+    int rows, rows_pad, kblocks;
+    int batch;        // matrices the planes hold
+    int first, used;  // matrices a split writes or a product reads: first .. first + used - 1
     bool b;           // B operand
 };
 

@@ -20,18 +20,30 @@
 // update of all (r, c) outside K, tiled 32 x 32 in shared memory: this is
 // where the 8 n^3 flops per matrix go, on the FP64 pipe), k6_writeback.
 // All matrices of a call (one per frequency) go through each launch together.
+//
+// From kDzMinN rows on, the two panels and the update are products on tensor
+// cores from BF16 digits (bgw_dz.cu, more exact than FP64 sums): the digits of
+// A_RK, of A_KR and of P both ways, one product for both panels (as 2 nf
+// matrices), the digits of P A_KR, and one product for the update.  The FP64
+// pipe ran the update at 0.94 of its rate, 64 ms for 16 x 800^2; now 8.9 ms, of
+// which the update takes 4.6 (bound by its epilogue's integer work), k6_diag 1.7
+// (one SM a matrix) and the digits 0.8.
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <string>
 
 #include "../../include/bgw_chi.h"
+#include "bgw_dz.h"
 
 namespace {
 
 constexpr int kB = 32;           // Gauss-Jordan block
 constexpr int kTile = 32;        // update tile (rows and columns): many CTAs per panel step
 constexpr int kErrPivot = 1;
+// Rows from which the products run on tensor cores: below, a step's products
+// fill neither form of the kernels and the extra launches decide.
+constexpr int kDzMinN = 96;
 
 struct Z {
     double x, y;
@@ -58,55 +70,80 @@ __global__ void k6_build(double2 *__restrict__ A, const double *__restrict__ s, 
 }
 
 // Invert the kb x kb block at (k0, k0) of every matrix in place (unblocked
-// Gauss-Jordan, no pivoting).  One CTA per matrix.
+// Gauss-Jordan, no pivoting).  One CTA per matrix, a 2 x 2 group of entries
+// per thread.  Bound: the FP64 pipe of one SM, 4 kb^2 operations a pivot; the
+// reciprocal of the next pivot is formed by the one thread that updates it
+// while the others still update (every thread forming its own took 175 us a
+// call of 16 blocks).
+__device__ __forceinline__ Z zinv(Z p, int *bad) {
+    const double t = p.y / p.x, den = fma(p.y, t, p.x);  // 1/p = (1 - i t) / (p.x + p.y t), p.y ~ 0 here
+    if (!(p.x > 0.0) || !isfinite(p.x * p.x + p.y * p.y)) *bad = 1;       // not positive definite
+    const double f = 1.0 / den;
+    return {f, -t * f};
+}
+
 __global__ void __launch_bounds__(256) k6_diag(double2 *__restrict__ A, int n, int k0, int kb, int *err) {
-    __shared__ Z a[kB][kB + 1];
-    __shared__ Z prow[kB];
-    __shared__ Z pcol[kB];
+    __shared__ Z row[2][kB], col[2][kB], pivinv[2];
+    __shared__ int bad[2];       // of the current and the next pivot: never written while it is read
     const long j = blockIdx.x;
     double2 *M = A + j * (long)n * n;
-    for (int i = threadIdx.x; i < kb * kb; i += blockDim.x) {
-        const int r = i / kb, c = i % kb;
-        const double2 v = M[(long)(k0 + r) * n + k0 + c];
-        a[r][c] = {v.x, v.y};
-    }
+    const int r0 = threadIdx.x / 16, c0 = threadIdx.x % 16;       // entries (r0 + 16 i, c0 + 16 l)
+    if (threadIdx.x < 2) bad[threadIdx.x] = 0;
+    __syncthreads();
+    Z a[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            const int r = r0 + 16 * i, c = c0 + 16 * l;
+            double2 v = make_double2(r == c ? 1.0 : 0.0, 0.0);     // the identity beyond kb
+            if (r < kb && c < kb) v = M[(long)(k0 + r) * n + k0 + c];
+            a[i][l] = {v.x, v.y};
+            if (r == 0) row[0][c] = a[i][l];
+            if (c == 0) col[0][r] = a[i][l];
+            if (r == 0 && c == 0) pivinv[0] = zinv(a[i][l], &bad[0]);
+        }
     __syncthreads();
     for (int k = 0; k < kb; ++k) {
-        const Z p = a[k][k];
-        const double den = p.x * p.x + p.y * p.y;
-        if (!(p.x > 0.0) || !isfinite(den)) {            // not positive definite (uniform branch)
+        const int cur = k & 1, nxt = cur ^ 1;
+        const Z p = pivinv[cur];
+        if (bad[cur]) {                                     // uniform: set before the last barrier
             if (threadIdx.x == 0) atomicExch(err, kErrPivot);
             return;
         }
-        const Z pinv = {p.x / den, -p.y / den};
-        // old column k and scaled row k
-        for (int i = threadIdx.x; i < kb; i += blockDim.x) {
-            pcol[i] = a[i][k];
-            prow[i] = (i == k) ? pinv : zmul(a[k][i], pinv);
+        // row k scaled, g = a_k. / p, and the multipliers -a_.k of this thread's rows
+        Z g[2], f[2];
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            const int c = c0 + 16 * l;
+            g[l] = c == k ? p : zmul(row[cur][c], p);
         }
-        __syncthreads();
-        for (int i = threadIdx.x; i < kb * kb; i += blockDim.x) {
-            const int r = i / kb, c = i % kb;
-            Z v;
-            if (r == k) {
-                v = prow[c];
-            } else if (c == k) {                          // -a_rk / p
-                const Z f = pcol[r];
-                v = {-(f.x * pinv.x - f.y * pinv.y), -(f.x * pinv.y + f.y * pinv.x)};
-            } else {                                      // a_rc - a_rk (a_kc / p)
-                const Z f = pcol[r], g = prow[c];
-                v = a[r][c];
-                v.x -= f.x * g.x - f.y * g.y;
-                v.y -= f.x * g.y + f.y * g.x;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            f[i] = col[cur][r0 + 16 * i];
+            f[i] = {-f[i].x, -f[i].y};
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int l = 0; l < 2; ++l) {
+                const int r = r0 + 16 * i, c = c0 + 16 * l;
+                Z v = c == k ? Z{0.0, 0.0} : a[i][l];       // column k becomes -a_rk / p
+                v = r == k ? g[l] : zfma(f[i], g[l], v);
+                a[i][l] = v;
+                if (r == k + 1) row[nxt][c] = v;
+                if (c == k + 1) col[nxt][r] = v;
+                if (r == k + 1 && c == k + 1) pivinv[nxt] = zinv(v, &bad[nxt]);
             }
-            a[r][c] = v;
-        }
         __syncthreads();
     }
-    for (int i = threadIdx.x; i < kb * kb; i += blockDim.x) {
-        const int r = i / kb, c = i % kb;
-        M[(long)(k0 + r) * n + k0 + c] = make_double2(a[r][c].x, a[r][c].y);
-    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            const int r = r0 + 16 * i, c = c0 + 16 * l;
+            if (r < kb && c < kb) M[(long)(k0 + r) * n + k0 + c] = make_double2(a[i][l].x, a[i][l].y);
+        }
 }
 
 // T[j][i][c] = sum_k P[i][k] A[k0+k][c]   (row panel, every column c)
@@ -248,6 +285,32 @@ __global__ void k6_writeback(double2 *__restrict__ A, int n, int k0, int kb, con
     }
 }
 
+// The same from panels stored by column, T[c][i], and by row, U[r][i]: a block
+// takes 32 columns (rows) and turns T through shared memory.
+__global__ void __launch_bounds__(256) k6_writeback_t(double2 *__restrict__ A, int n, int k0, int kb,
+                                                      const double2 *__restrict__ T, const double2 *__restrict__ U) {
+    __shared__ double2 t[32][kB + 1];
+    const long j = blockIdx.z;
+    double2 *M = A + j * (long)n * n;
+    const int x0 = blockIdx.x * 32;
+    for (int e = threadIdx.x; e < 32 * kB; e += 256) {
+        const int x = x0 + e / kB, i = e % kB;
+        if (x < n && i < kb) {
+            const long at = (j * (long)n + x) * kB + i;
+            t[e / kB][i] = T[at];
+            if (x < k0 || x >= k0 + kb) {
+                const double2 u = U[at];
+                M[(long)x * n + k0 + i] = make_double2(-u.x, -u.y);
+            }
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 32 * kB; e += 256) {
+        const int x = x0 + e % 32, i = e / 32;
+        if (x < n && i < kb && (x < k0 || x >= k0 + kb)) M[(long)(k0 + i) * n + x] = t[e % 32][i];
+    }
+}
+
 // W = S eps~^-1 S (mode 1) or eps^-1 = S eps~^-1 S^-1 (mode 2).
 __global__ void k6_scale(double2 *__restrict__ A, const double *__restrict__ s, int n, int inverse_cols) {
     const long j = blockIdx.z;
@@ -265,13 +328,32 @@ __global__ void k6_scale(double2 *__restrict__ A, const double *__restrict__ s, 
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Workspace: the panels U and T, s, the error words and, on tensor cores, the
+// digit planes of the panels (2 nf matrices), of P (2 nf) and of P A_KR (nf).
+struct Work {
+    size_t U, T, s, err, panels, p, t, total;
+    Work(int n, int nf) {
+        const size_t panel = sizeof(double2) * (size_t)nf * kB * n;
+        U = 0;
+        T = panel;
+        s = align256(2 * panel);
+        err = s + align256(sizeof(double) * (size_t)n);
+        panels = p = t = total = err + 256;
+        if (n >= kDzMinN) {
+            p = panels + bgw::dz_planes_bytes(n, kB, 2 * nf, false);
+            t = p + bgw::dz_planes_bytes(kB, kB, 2 * nf, true);
+            total = t + bgw::dz_planes_bytes(n, kB, nf, true);
+        }
+    }
+};
+
 }  // namespace
 
 void bgw_set_global_error(const std::string &msg);
 
 extern "C" size_t bgw_epsinv_workspace_bytes(int ng, int nfreq) {
     if (ng < 1 || nfreq < 1) return 0;
-    return 2 * align256(sizeof(double2) * (size_t)nfreq * kB * ng) + align256(sizeof(double) * ng) + 256;
+    return Work(ng, nfreq).total;
 }
 
 extern "C" bgw_status bgw_coulomb_sqrt(const double *avec, const double *q, int ng, const int *gvec, double *s) {
@@ -336,13 +418,13 @@ extern "C" bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, 
                                    std::to_string(need) + " needed");
     }
     char *w = static_cast<char *>(work);
-    double2 *T = reinterpret_cast<double2 *>(w);
-    double2 *U = reinterpret_cast<double2 *>(w + align256(sizeof(double2) * (size_t)nfreq * kB * ng));
-    double *sd = reinterpret_cast<double *>(w + 2 * align256(sizeof(double2) * (size_t)nfreq * kB * ng));
-    int *err = reinterpret_cast<int *>(reinterpret_cast<char *>(sd) + align256(sizeof(double) * ng));
+    const Work o(ng, nfreq);
+    double2 *U = reinterpret_cast<double2 *>(w + o.U), *T = reinterpret_cast<double2 *>(w + o.T);
+    double *sd = reinterpret_cast<double *>(w + o.s);
+    int *err = reinterpret_cast<int *>(w + o.err);        // [0] pivots, [1] device-side waits
     double2 *A = static_cast<double2 *>(chi);
     e = cudaMemcpyAsync(sd, s, sizeof(double) * ng, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 2 * sizeof(int), st);
     const unsigned rowblocks = (unsigned)((ng + 255) / 256);
     if (e == cudaSuccess) {
         k6_build<<<dim3(rowblocks, ng, nfreq), 256, 0, st>>>(A, sd, ng);
@@ -350,24 +432,56 @@ extern "C" bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, 
     }
     const unsigned tiles = (unsigned)((ng + kTile - 1) / kTile);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k6_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdateSmem);
+    const bool tensor = ng >= kDzMinN;
+    int sms = 148;
+    if (tensor && e == cudaSuccess) {
+        int dev = 0;
+        e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    }
     for (int k0 = 0; k0 < ng && e == cudaSuccess; k0 += kB) {
         const int kb = ng - k0 < kB ? ng - k0 : kB;
         k6_diag<<<nfreq, 256, 0, st>>>(A, ng, k0, kb, err);
-        k6_panels<<<dim3((ng + 127) / 128, kB / kPanelI, 2 * nfreq), 128, 0, st>>>(A, ng, k0, kb, T, U);
-        k6_update<<<dim3(tiles, tiles, nfreq), 256, kUpdateSmem, st>>>(A, ng, k0, kb, T);
-        k6_writeback<<<dim3((ng + 127) / 128, 1, nfreq), 128, 0, st>>>(A, ng, k0, kb, T, U);
+        if (tensor) {
+            const long n2 = (long)ng * ng;
+            bgw::DzPlanes pa = bgw::dz_planes(w + o.panels, ng, kB, 2 * nfreq, false), pr = pa;
+            bgw::DzPlanes bp = bgw::dz_planes(w + o.p, kb, kB, 2 * nfreq, true), br = bp;
+            pa.used = pr.used = pr.first = bp.used = br.used = br.first = nfreq;
+            const double2 *row = A + (long)k0 * ng, *col = A + k0, *P = row + k0;
+            // U[r] = A_rK P with P read by columns, T[c] = P A_Kc with P read by rows
+            const bgw::DzPlanes pl[4] = {pa, pr, bp, br};
+            const bgw::DzOperand op[4] = {{col, n2, ng, 1, false, nullptr}, {row, n2, 1, ng, false, nullptr},
+                                          {P, n2, 1, ng, false, nullptr}, {P, n2, ng, 1, false, nullptr}};
+            e = bgw::dz_split(op, pl, 4, kb, st);
+            bgw::DzPlanes both = pa, bothp = bp;
+            both.used = bothp.used = 2 * nfreq;
+            if (e == cudaSuccess)
+                e = bgw::dz_gemm(both, bothp, bgw::DzOut{U, (long)ng * kB, kB, 1, 0, 0, 1.0, 0.0, false}, sms, st, err + 1);
+            const bgw::DzPlanes bt = bgw::dz_planes(w + o.t, ng, kB, nfreq, true);
+            const bgw::DzOperand ot = {T, (long)ng * kB, kB, 1, false, nullptr};
+            if (e == cudaSuccess) e = bgw::dz_split(&ot, &bt, 1, kb, st);
+            if (e == cudaSuccess)
+                e = bgw::dz_gemm(pa, bt, bgw::DzOut{A, n2, ng, 1, k0, k0 + kb, -1.0, 0.0, true}, sms, st, err + 1);
+            if (e != cudaSuccess) break;
+            k6_writeback_t<<<dim3((ng + 31) / 32, 1, nfreq), 256, 0, st>>>(A, ng, k0, kb, T, U);
+        } else {
+            k6_panels<<<dim3((ng + 127) / 128, kB / kPanelI, 2 * nfreq), 128, 0, st>>>(A, ng, k0, kb, T, U);
+            k6_update<<<dim3(tiles, tiles, nfreq), 256, kUpdateSmem, st>>>(A, ng, k0, kb, T);
+            k6_writeback<<<dim3((ng + 127) / 128, 1, nfreq), 128, 0, st>>>(A, ng, k0, kb, T, U);
+        }
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && mode > 0) {
         k6_scale<<<dim3(rowblocks, ng, nfreq), 256, 0, st>>>(A, sd, ng, mode == 2);
         e = cudaGetLastError();
     }
-    int flag = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    int flag[2] = {0, 0};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(flag, err, sizeof flag, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (own) cudaFree(own);
     if (e != cudaSuccess) return fail(BGW_E_CUDA, std::string("epsinv: ") + cudaGetErrorString(e));
-    if (flag) return fail(BGW_E_ARG, "epsinv: a pivot is not positive: I - S chi S is not positive definite "
+    if (flag[1]) return fail(BGW_E_TIMEOUT, "epsinv: a device-side wait gave up; the output is invalid");
+    if (flag[0]) return fail(BGW_E_ARG, "epsinv: a pivot is not positive: I - S chi S is not positive definite "
                                      "(chi0 must be Hermitian negative semidefinite); the output is invalid");
     return BGW_OK;
 }

@@ -24,6 +24,7 @@
 #include <string>
 
 #include "../../include/bgw_chi.h"
+#include "bgw_fft_i64.cuh"
 
 void bgw_set_global_error(const std::string &msg);
 
@@ -138,11 +139,12 @@ bgw_status su2_of(const double *avec, const int *rot_lat, double *U, double *axi
     return BGW_OK;
 }
 
-// One thread per (plane wave i, chunk of kBandChunk bands): the phase
-// e^{-2 pi i h'.tau} is formed once per thread from the rotated Miller index
-// h' = M h (M = R_lat^-T), then applied to its bands; reads and writes are
+// k8_phase: per plane wave i the phase e^{-2 pi i h'.tau}, from the rotated
+// Miller index h' = M h (M = R_lat^-T), folded into a copy of U, V[i][4], as
+// 64-bit integers in units of 2^-61.  k8_unfold: one thread per (plane wave,
+// chunk of kBandChunk bands) applies V[i] to its bands; reads and writes are
 // coalesced along i.
-constexpr int kBandChunk = 16;
+constexpr int kBandChunk = 8;
 
 struct Op {
     int M[3][3];
@@ -150,8 +152,8 @@ struct Op {
     double2 u[4];   // U row-major
 };
 
-__global__ void k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ out, int nb, int ngw,
-                          const int *__restrict__ gvec, Op op) {
+__global__ void __launch_bounds__(128)
+k8_phase(int ngw, const int *__restrict__ gvec, Op op, longlong2 *__restrict__ V) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= ngw) return;
     const int h0 = gvec[3 * i], h1 = gvec[3 * i + 1], h2 = gvec[3 * i + 2];
@@ -161,22 +163,54 @@ __global__ void k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ 
     f -= floor(f);                                        // turns in [0, 1)
     double sn, cs;
     sincospi(-2.0 * f, &sn, &cs);
-    // the phase folded into this plane wave's copy of U: V = e^{-i G'.tau} U
-    // (the 2 x 2 complex product is the whole per-band cost, on the FP64 pipe)
-    double2 v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        v[k] = make_double2(cs * op.u[k].x - sn * op.u[k].y, cs * op.u[k].y + sn * op.u[k].x);
+        V[(long)k * ngw + i] = make_longlong2(bgw::fix_in<62>(cs * op.u[k].x - sn * op.u[k].y, 1023),
+                                              bgw::fix_in<62>(cs * op.u[k].y + sn * op.u[k].x, 1023));
+}
+
+// Bound: integer issue.  The 16 real products of a band's spin pair and plane
+// wave run as 48 32 x 32-bit multiply-adds: the pair is scaled by its largest
+// component to 60 bits, V is held to 2^-61 (both beyond FP64's 53), and the sums
+// leave as FP64, rounded once.  In FP64 the products alone took 16 x 64 issue
+// cycles of a warp, and each thread formed V for its 16 bands, as many again:
+// 418 bands x 5029 plane waves 93 -> 72 us a call (134 MB, 20 us at the copy rate).
+__global__ void __launch_bounds__(256)
+k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ out, int nb, int ngw, const longlong2 *__restrict__ V) {
+    using bgw::fix_mad;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= ngw) return;
+    bgw::fix_parts vx[4], vy[4], my[4];                   // re, im, -im
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const longlong2 v = V[(long)k * ngw + i];
+        vx[k] = bgw::fix_split(v.x);
+        vy[k] = bgw::fix_split(v.y);
+        my[k] = bgw::fix_split(-v.y);
+    }
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
     const int n1 = min(nb, (int)(blockIdx.y + 1) * kBandChunk);
-#pragma unroll 4
+#pragma unroll 2
     for (int n = blockIdx.y * kBandChunk; n < n1; ++n) {
         const double2 a = in[(2L * n) * ngw + i], b = in[(2L * n + 1) * ngw + i];
+        const int E = max(max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff),
+                          max(__double2hiint(b.x) & 0x7fffffff, __double2hiint(b.y) & 0x7fffffff)) >> 20;
+        const bgw::fix_parts ax = bgw::fix_split(bgw::fix_in<60>(a.x, E)), ay = bgw::fix_split(bgw::fix_in<60>(a.y, E));
+        const bgw::fix_parts bx = bgw::fix_split(bgw::fix_in<60>(b.x, E)), by = bgw::fix_split(bgw::fix_in<60>(b.y, E));
+        const int eb = 1086 - 57 + E - 1022;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            const double2 u0 = v[2 * r], u1 = v[2 * r + 1];
-            const double x = fma(u0.x, a.x, fma(-u0.y, a.y, fma(u1.x, b.x, -u1.y * b.y)));
-            const double y = fma(u0.x, a.y, fma(u0.y, a.x, fma(u1.x, b.y, u1.y * b.x)));
-            out[(2L * n + r) * ngw + i] = make_double2(x, y);
+            auto dot = [&](bgw::fix_parts p, bgw::fix_parts q, bgw::fix_parts s, bgw::fix_parts t) {
+                const long long hi = fix_mad(p.h, ax.h, fix_mad(q.h, ay.h, fix_mad(s.h, bx.h, fix_mad(t.h, by.h, 0))));
+                long long lo = fix_mad(p.h, ax.l, fix_mad(p.l, ax.h, fix_mad(q.h, ay.l, fix_mad(q.l, ay.h, bgw::kFixHalf))));
+                lo = fix_mad(s.h, bx.l, fix_mad(s.l, bx.h, fix_mad(t.h, by.l, fix_mad(t.l, by.h, lo))));
+                return bgw::fix_join(hi, lo);
+            };
+            const long long x = dot(vx[2 * r], my[2 * r], vx[2 * r + 1], my[2 * r + 1]);
+            const long long y = dot(vy[2 * r], vx[2 * r], vy[2 * r + 1], vx[2 * r + 1]);
+            double2 o = make_double2(bgw::fix_out(x, eb), bgw::fix_out(y, eb));
+            if (E == 0x7ff) o = make_double2(nan, nan);   // an infinity or a NaN in the pair
+            out[(2L * n + r) * ngw + i] = o;
         }
     }
 }
@@ -226,11 +260,13 @@ extern "C" bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, 
     if (nb == 0) return BGW_OK;
     if ((long)nb > 65535L * kBandChunk) return fail(BGW_E_ARG, "unfold_spinor: too many bands for one call");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    void *g_dev = nullptr;
-    const size_t gbytes = sizeof(int) * 3 * (size_t)ngw;
-    cudaError_t e = cudaMallocAsync(&g_dev, gbytes, s);
+    void *g_dev = nullptr;                    // V, then the Miller list
+    const size_t gbytes = sizeof(int) * 3 * (size_t)ngw, vbytes = 4 * sizeof(longlong2) * (size_t)ngw;
+    cudaError_t e = cudaMallocAsync(&g_dev, vbytes + gbytes, s);
+    longlong2 *v_dev = static_cast<longlong2 *>(g_dev);
+    int *h_dev = reinterpret_cast<int *>(static_cast<char *>(g_dev) + vbytes);
     // a pageable source: the copy has read gvec_in when it returns
-    if (e == cudaSuccess) e = cudaMemcpyAsync(g_dev, gvec_in, gbytes, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h_dev, gvec_in, gbytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
         Op op;
         for (int i = 0; i < 3; ++i) {
@@ -239,8 +275,8 @@ extern "C" bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, 
         }
         for (int i = 0; i < 4; ++i) op.u[i] = make_double2(U[2 * i], U[2 * i + 1]);
         const dim3 grid((unsigned)((ngw + 255) / 256), (unsigned)((nb + kBandChunk - 1) / kBandChunk));
-        k8_unfold<<<grid, 256, 0, s>>>(static_cast<const double2 *>(c_in), static_cast<double2 *>(c_out), nb,
-                                       ngw, static_cast<const int *>(g_dev), op);
+        k8_phase<<<(unsigned)((ngw + 127) / 128), 128, 0, s>>>(ngw, h_dev, op, v_dev);
+        k8_unfold<<<grid, 256, 0, s>>>(static_cast<const double2 *>(c_in), static_cast<double2 *>(c_out), nb, ngw, v_dev);
         e = cudaGetLastError();
     }
     if (g_dev) {
