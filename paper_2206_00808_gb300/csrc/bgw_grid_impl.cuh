@@ -352,69 +352,88 @@ k2_zpass_c4(const C *__restrict__ Uv, const C *__restrict__ Uc, int nc, long P, 
 // Threads of the eight-lane kernels below: 32 groups of eight lanes.
 constexpr int kOctThreads = 256;
 
-// Pair density + z and y forward passes of one (pair, x-plane) per CTA for
-// the eight-lane lengths (48, 64): group y of eight lanes forms the pair
-// density of z line y from the grids (both spin components) and transforms
-// it (fft_line_oct); the kept w2 outputs go to shared Zs[N][w2p]; then group
-// jz transforms y line jz of Zs and writes the kept w1 outputs to
-// Bs[p][x][w1][w2].  The z-pass output never leaves the SM.  Each group has
-// its own 8 x 9 exchange block after Zs.  Lane t handles z = 8m + t on the
-// way in and the outputs f = t + (N/8) k1 on the way out.  A warp whose four
-// groups all lie past the last line skips the iteration (the lanes of a warp
-// synchronise inside the transform).  Three CTAs per SM (80 registers) hide
-// the latency of the grid loads.  grid (P, n0).
-template <int N>
-__global__ void __launch_bounds__(kOctThreads, 3)
+// Pair density + z and y forward passes of one x-plane and up to TC pairs of
+// one valence band per CTA for the eight-lane lengths (48, 64): group y of
+// eight lanes reads z line y of the valence band once, forms the pair density
+// with each conduction band from the grids (both spin components) and
+// transforms it (fft_line_oct); the kept w2 outputs go to shared
+// Zs[pair][N][w2p]; then group (pair, jz) transforms y line jz of its Zs and
+// writes the kept w1 outputs to Bs[p][x][w1][w2].  The z-pass output never
+// leaves the SM.  Each group has its own 8 x 9 exchange block after Zs.  Lane t
+// handles z = 8m + t on the way in and the outputs f = t + (N/8) k1 on the way
+// out.  A warp whose four groups all lie past the last line skips the iteration
+// (the lanes of a warp synchronise inside the transform).  Bound: the grids
+// come from L2, four planes a pair with one pair per CTA (4.5 TB/s at 64^3);
+// with TC pairs it is 2 + 2/TC, and the TC w2 y lines fill the groups better.
+// Measured (FP32 64^3, 8 x 125 pairs of 2 k-points, w2 = 29): 3.74 -> 3.05 ms;
+// reading the next band's planes during a transform did not help (3.12).
+// grid (nv ceil(nc / TC), n0).
+template <int N, int TC>
+__global__ void __launch_bounds__(kOctThreads, TC == 1 ? 3 : 2)
 k2_zy_oct(const C *__restrict__ Uv, const C *__restrict__ Uc, int nc, int w1, int w2, int s1, int s2,
           C *__restrict__ Bs) {
     extern __shared__ unsigned char zy_sm[];
     constexpr int M = N / 8, G = kOctThreads / 8;      // groups per CTA
     const int w2p = w2 | 1;
+    const int ZP = (N * w2p + 1) & ~1;                   // one pair's z outputs
     C *Zs = reinterpret_cast<C *>(zy_sm);
     const int grp = threadIdx.x >> 3, t = threadIdx.x & 7;
-    C *ex = Zs + ((N * w2p + 1) & ~1) + grp * kOctBlock;
+    C *ex = Zs + TC * ZP + grp * kOctBlock;
     const int warp_first_grp = (threadIdx.x >> 5) * 4;
     C tw[M];
     oct_twiddles<T, -1, N>(t, tw);
-    const long p = blockIdx.x;
     const int x = blockIdx.y, n0 = gridDim.y;
-    const long v = p / nc, c = p % nc;
+    const int cgroups = (nc + TC - 1) / TC;
+    const long v = blockIdx.x / cgroups;
+    const int c0 = (int)(blockIdx.x % cgroups) * TC, tc = min(TC, nc - c0);
     const long plane = (long)N * N, vol = (long)n0 * plane;
     const C *pv = Uv + (2 * v) * vol + x * plane;
-    const C *pc = Uc + (2 * c) * vol + x * plane;
+    const C *pc = Uc + 2L * c0 * vol + x * plane;
     const int ns2 = N - s2, ns1 = N - s1;
     for (int y0 = 0; y0 < N; y0 += G) {
         if (y0 + warp_first_grp >= N) break;            // warp-uniform
         const int y = y0 + grp;
         const bool valid = y < N;
         const long row = (long)(valid ? y : 0) * N;
-        C a[M], out[8];
+        C va[M], vb[M];
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            const long o = row + 8 * m + t;
-            a[m] = rho2(pv[o], pc[o], pv[vol + o], pc[vol + o]);
+            va[m] = pv[row + 8 * m + t];
+            vb[m] = pv[vol + row + 8 * m + t];
         }
-        fft_line_oct<T, -1, N>(a, t, ex, tw, out);
-        if (valid && t < M) {
+#pragma unroll 1
+        for (int c = 0; c < tc; ++c) {
+            const C *pcc = pc + 2L * c * vol;
+            C a[M], out[8];
 #pragma unroll
-            for (int k1 = 0; k1 < 8; ++k1) {
-                const int jj = rot<N>(t + M * k1, ns2);
-                if (jj < w2) Zs[y * w2p + jj] = out[k1];
+            for (int m = 0; m < M; ++m) {
+                const long o = row + 8 * m + t;
+                a[m] = rho2(va[m], pcc[o], vb[m], pcc[vol + o]);
+            }
+            fft_line_oct<T, -1, N>(a, t, ex, tw, out);
+            if (valid && t < M) {
+#pragma unroll
+                for (int k1 = 0; k1 < 8; ++k1) {
+                    const int jj = rot<N>(t + M * k1, ns2);
+                    if (jj < w2) Zs[c * ZP + y * w2p + jj] = out[k1];
+                }
             }
         }
     }
     __syncthreads();
-    for (int base = 0; base < w2; base += G) {
-        if (base + warp_first_grp >= w2) break;          // warp-uniform
-        const int jz = base + grp;
-        const bool valid = jz < w2;
-        const int jc = valid ? jz : 0;
+    const int lines = tc * w2;
+    for (int base = 0; base < lines; base += G) {
+        if (base + warp_first_grp >= lines) break;       // warp-uniform
+        const int l = base + grp;
+        const bool valid = l < lines;
+        const int c = valid ? l / w2 : 0, jz = valid ? l % w2 : 0;
+        const C *zi = Zs + c * ZP + jz;
         C a[M], out[8];
 #pragma unroll
-        for (int m = 0; m < M; ++m) a[m] = Zs[(8 * m + t) * w2p + jc];
+        for (int m = 0; m < M; ++m) a[m] = zi[(8 * m + t) * w2p];
         fft_line_oct<T, -1, N>(a, t, ex, tw, out);
         if (valid && t < M) {
-            C *bo = Bs + ((p * n0 + x) * w1) * w2 + jz;
+            C *bo = Bs + (((v * nc + c0 + c) * n0 + x) * w1) * (long)w2 + jz;
 #pragma unroll
             for (int k1 = 0; k1 < 8; ++k1) {
                 const int jj = rot<N>(t + M * k1, ns1);
@@ -1525,15 +1544,21 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
     const long P = (long)nv * nc;
     if (oct_len(a) && (lanes == 8 || (lanes == 0 && use_coop(a) && use_oct(a)))) {
         // eight lanes per line: fused z+y, then the x pass
-        const size_t zs = sizeof(C) * ((((size_t)a.n[1] * (a.w[2] | 1)) + 1) / 2 * 2 +
-                                       (size_t)(kOctThreads / 8) * kOctBlock);
         cudaError_t e = cudaSuccess;
+        // pairs per CTA: as many of 4, 2, 1 as leave two CTAs per SM and do not
+        // leave SMs without one
+        const size_t ex = sizeof(C) * (size_t)(kOctThreads / 8) * kOctBlock;
+        const size_t zp = sizeof(C) * ((((size_t)a.n[1] * (a.w[2] | 1)) + 1) / 2 * 2);
+        int tcs = 4;
+        while (tcs > 1 && (ex + tcs * zp > (size_t)110 * 1024 || nc < tcs)) tcs /= 2;
+        const size_t zs = ex + tcs * zp;
         BGW_FOR_EACH_OCT_LEN(a.n[2], {
+            auto kern = tcs == 4 ? k2_zy_oct<N, 4> : tcs == 2 ? k2_zy_oct<N, 2> : k2_zy_oct<N, 1>;
             if (zs > 48 * 1024) {
-                e = cudaFuncSetAttribute(k2_zy_oct<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zs);
+                e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zs);
                 if (e != cudaSuccess) return e;
             }
-            k2_zy_oct<N><<<dim3((unsigned)P, (unsigned)a.n[0]), kOctThreads, zs, st>>>(
+            kern<<<dim3((unsigned)(nv * ((nc + tcs - 1) / tcs)), (unsigned)a.n[0]), kOctThreads, zs, st>>>(
                 uv, uc, nc, a.w[1], a.w[2], a.s[1], a.s[2], Bp);
         });
         const long lines = (long)a.w[1] * a.w[2];
