@@ -25,8 +25,8 @@
 // Kernels:
 //   k5z_rowmax  per frequency and row, max_p |Y| in FP32 (an upper bound
 //               with margin), merged across blocks by atomicMax on float bits
-//   k5z_split   Y in FP64, N by the 1.5 * 2^52 rounding constant, the digits
-//               by integer shifts; the five planes per frequency stored as
+//   k5z_split   N from the integer product of the mantissas, the digits by
+//               integer shifts; the five planes per frequency stored as
 //               tiles [R/128][Kp/32][128 rows][32 pairs] of BF16 (64-byte rows)
 //   k5z_gemm    persistent, one CTA per SM over (lower 128 x 64 tile of D,
 //               frequency) items: warp 8 issues TMA loads (64-byte swizzle; the
@@ -45,6 +45,7 @@
 #include <cstring>
 
 #include "bgw_f64tc.h"
+#include "bgw_fft_i64.cuh"
 #include "bgw_tc_common.cuh"
 
 namespace bgw {
@@ -69,7 +70,8 @@ constexpr int kErrFull = 1, kErrEmpty = 2, kErrAccum = 3, kErrDrain = 4;
 constexpr int kErrSign = F64TC_ERR_SIGN;      // a pair weight > 0 (see f64tc_contract)
 
 // ---------------------------------------------------------- row maxima --
-constexpr int kRmP = 256, kRmG = 32, kRmF = 16;
+// 64 pairs per block: 1600 pairs of 350 G are 275 blocks (77 with 256)
+constexpr int kRmP = 64, kRmG = 32, kRmF = 16;
 
 __global__ void __launch_bounds__(256)
 k5z_rowmax(const double2 *__restrict__ M, int P, int ng, const double *__restrict__ w, int nfreq, int R,
@@ -140,11 +142,29 @@ __device__ __forceinline__ int row_exponent(unsigned mb) {
     return k + 1;
 }
 
-// Signed base-256 digits of N = rint(y sc), |N| <= 2^39 (1 + 2^-20):
-// N = d0 2^32 + d1 2^24 + d2 2^16 + d3 2^8 + d4, every |d_t| <= 128.
-__device__ __forceinline__ void digits(double y, double sc, int (&d)[kSl]) {
-    const double magic = 6755399441055744.0;   // 1.5 * 2^52: fma rounds y sc to an integer
-    long long n = __double_as_longlong(fma(y, sc, magic)) - __double_as_longlong(magic);
+// y = sqrt(-w) m as an integer: the mantissas (53 bits, at the top of 63) of
+// both factors multiply to 62 bits, and a shift rounds to N = rint(y 2^(40-e)),
+// |N| <= 2^39 (1 + 2^-20).  In FP64 the product and the rounding took two thirds
+// of k5z_split (a warp's FP64 operation holds its scheduler 64 cycles, this some 30).
+struct Mant {
+    int h, l;      // signed halves of mantissa 2^9: value = (h 2^32 + l) 2^(e - 1084)
+    int e;         // biased exponent (0: zero)
+};
+__device__ __forceinline__ Mant mant(double v) {
+    const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+    unsigned long long m = (((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v)) << 9;
+    if (e == 0) m = 0;
+    const long long s = (long long)m;
+    const fix_parts p = fix_split(hi < 0 ? -s : s);
+    return {p.h, p.l, e};
+}
+// Signed base-256 digits of N = d0 2^32 + d1 2^24 + d2 2^16 + d3 2^8 + d4,
+// every |d_t| <= 128; sh = 40 - e of the row.
+__device__ __forceinline__ void digits(const Mant &a, const Mant &b, int sh, int (&d)[kSl]) {
+    // x y = q 2^64 2^(a.e + b.e - 2168) with q = the top 64 bits of the product (|q| <= 2^60)
+    const long long q = fix_join(fix_mad(a.h, b.h, 0), fix_mad(a.h, b.l, fix_mad(a.l, b.h, kFixHalf)));
+    const int r = max(1, 2104 - a.e - b.e - sh);          // N = rint(q 2^-r), r >= 18 wherever |N| <= 2^39
+    long long n = r >= 62 ? 0 : (q + (1LL << (r - 1))) >> r;
     d[0] = (int)((n + (1LL << 31)) >> 32);
     n -= (long long)d[0] << 32;
     d[1] = (int)((n + (1LL << 23)) >> 24);
@@ -164,7 +184,7 @@ __global__ void __launch_bounds__(256)
 k5z_split(const double2 *__restrict__ M, int P, int ng, const double *__restrict__ w, int nfreq, int R, int Kp,
           const unsigned *__restrict__ rmax, int *__restrict__ rexp, __nv_bfloat16 *__restrict__ X) {
     __shared__ double2 sm[kSpP][kSpG + 1];
-    __shared__ double ss[kSpP];
+    __shared__ Mant ss[kSpP];
     const int p0 = blockIdx.x * kSpP, g0 = blockIdx.y * kSpG;
     for (int i = threadIdx.x; i < kSpP * kSpG; i += 256) {
         const int pp = i / kSpG, gg = i % kSpG;
@@ -177,25 +197,30 @@ k5z_split(const double2 *__restrict__ M, int P, int ng, const double *__restrict
     const long kblocks = Kp / kKB;
     const long planeElems = (long)R * Kp;
     __nv_bfloat16 *base = X + (((long)(row / kM) * kblocks + p0 / kKB) * kM + row % kM) * kKB + pq;
+    __syncthreads();
+    Mant mv[8];                                 // this thread's values of M, for every frequency
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const double2 m = sm[pq + i][r >> 1];
+        mv[i] = mant((r & 1) ? m.y : m.x);
+    }
     const float dscale[kSl] = {1.0f, 0x1p-8f, 0x1p-16f, 0x1p-24f, 0x1p-32f};
     for (int j = 0; j < nfreq; ++j) {
         __syncthreads();
         if (threadIdx.x < kSpP) {
             const int p = p0 + threadIdx.x;
             const double wv = p < P ? w[(long)j * P + p] : 0.0;
-            ss[threadIdx.x] = wv < 0.0 ? sqrt(-wv) : 0.0;
+            ss[threadIdx.x] = mant(wv < 0.0 ? sqrt(-wv) : 0.0);
         }
         __syncthreads();
         const int e = row_exponent(rmax[(long)j * R + row]);
         if (blockIdx.x == 0 && (threadIdx.x % 4) == 0) rexp[(long)j * R + row] = e;
-        const double sc = __longlong_as_double((long long)(1023 + 40 - e) << 52);   // 2^(40-e)
         uint32_t h[kSl][4];
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {
-            const double2 ma = sm[pq + i][r >> 1], mb = sm[pq + i + 1][r >> 1];
             int da[kSl], db[kSl];
-            digits(ss[pq + i] * ((r & 1) ? ma.y : ma.x), sc, da);
-            digits(ss[pq + i + 1] * ((r & 1) ? mb.y : mb.x), sc, db);
+            digits(ss[pq + i], mv[i], 40 - e, da);
+            digits(ss[pq + i + 1], mv[i + 1], 40 - e, db);
 #pragma unroll
             for (int t = 0; t < kSl; ++t)
                 h[t][i / 2] = bf2_bits(__floats2bfloat162_rn((float)da[t] * dscale[t], (float)db[t] * dscale[t]));
