@@ -169,6 +169,8 @@ struct bgw_ctx_s {
     DevBuf freq_dev;
     DevBuf out_stage;    // finalize to host
     DevBuf gmap_tmp;     // dielectric-sphere map of a bgw_mtxel_spinor call
+    std::vector<int> gmap_host;      // its contents, while every write of it is known (see put_gmap)
+    bool gmap_captured = false;
     DevBuf errflag;      // device int: non-zero after a bounded device wait gave up
     // scratch of the self-energy and BSE kernel calls (matrix-element blocks,
     // products, per-pair sums, a copy of the interaction's diagonal)
@@ -571,6 +573,23 @@ cudaError_t ensure_mtxel_scratch(bgw_ctx_s *c, const QState &s, int na, int nb2)
     return e;
 }
 
+// The call's dielectric-sphere map into gmap_tmp; nothing is copied when it
+// holds these very values already (a third of a small call's host time).  Once
+// a copy has been captured in a graph, its replays write the buffer behind the
+// library's back and every call copies.
+cudaError_t put_gmap(bgw_ctx_s *c, const std::vector<int> &gmap) {
+    if (st_capturing(c)) c->gmap_captured = true;
+    if (!c->gmap_captured && c->gmap_tmp.p && c->gmap_host == gmap) return cudaSuccess;
+    c->gmap_host.clear();
+    cudaError_t e = c->gmap_tmp.ensure(sizeof(int) * gmap.size(), c->st);
+    // a pageable source: the copy is stream-ordered and has read the vector
+    // when it returns, so the buffer can be refilled by a later call
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->gmap_tmp.p, gmap.data(), sizeof(int) * gmap.size(), cudaMemcpyHostToDevice, c->st);
+    if (e == cudaSuccess && !c->gmap_captured) c->gmap_host = gmap;
+    return e;
+}
+
 // Profiling of the matrix-element kernels in two stages: 1 the pair density
 // with the z and y passes, 6 the x pass with the sphere gather.  The hook
 // closes the open record and opens one of the other stage at each x-pass mark.
@@ -943,12 +962,8 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
     if (e != cudaSuccess) return c->cuda_fail(e, "deferred sphere-to-grid kernels");
     e = ensure_mtxel_scratch(c, s, na, nb2);
     if (e != cudaSuccess) return c->cuda_fail(e, "matrix-element scratch");
-    e = c->gmap_tmp.ensure(sizeof(int) * s.gmap.size(), c->st);
+    e = put_gmap(c, s.gmap);
     if (e != cudaSuccess) return c->cuda_fail(e, "map buffer");
-    // pageable source: the copy is stream-ordered and has read the host
-    // vector when it returns, so the buffer can be refilled by a later call
-    e = cudaMemcpyAsync(c->gmap_tmp.p, s.gmap.data(), sizeof(int) * s.gmap.size(), cudaMemcpyHostToDevice, c->st);
-    if (e != cudaSuccess) return c->cuda_fail(e, "map copy");
     const bgw::Axes ax = mtxel_axes(c, s, G0);
     cudaError_t ge;
     const int sa = ensure_grid(c, ik, ge);
@@ -1316,13 +1331,8 @@ bgw_status bgw_mtxel_spinor(bgw_ctx c, const bgw_q *q, int ik, int v0, int nv, i
     if (e != cudaSuccess) return c->cuda_fail(e, "mtxel: deferred sphere-to-grid kernels");
     e = ensure_mtxel_scratch(c, s, nv, nc);
     if (e != cudaSuccess) return c->cuda_fail(e, "mtxel: scratch");
-    // The per-call map goes to a context buffer; reuse is stream-ordered and
-    // a pageable-memory copy has read the host vector when the call returns.
-    e = c->gmap_tmp.ensure(sizeof(int) * s.gmap.size(), c->st);
+    e = put_gmap(c, s.gmap);
     if (e != cudaSuccess) return c->cuda_fail(e, "mtxel: map buffer");
-    e = cudaMemcpyAsync(c->gmap_tmp.p, s.gmap.data(), sizeof(int) * s.gmap.size(), cudaMemcpyHostToDevice,
-                        c->st);
-    if (e != cudaSuccess) return c->cuda_fail(e, "mtxel: map copy");
     s.gmap_dev.p = c->gmap_tmp.p;   // borrowed, not owned
     e = launch_mtxel(c, s, ik, kp, G0, v0, nv, c0, nc, M_dev, s.ng);
     s.gmap_dev.p = nullptr;

@@ -29,3 +29,25 @@ def test_mtxel_block_matches_oracle(gpu_lib, prec, v0, nv, c0, nc):
     gpu_lib.bgw_mtxel_spinor(ctx.ctx, q, geps, ik, v0, nv, c0, nc, M)
     ctx.close()
     assert np.abs(M.cpu().numpy() - ref).max() <= TOL_M[prec] * np.abs(ref).max()
+
+
+def test_alternating_spheres(gpu_lib):
+    """The sphere map is copied to the device only when it changes: the same
+    sphere twice, another of the same size, then the first again."""
+    torch = pytest.importorskip("torch")
+    p = syn.make_problem("si18_qx", nv=2, nc=3)
+    q, a, _ = p.qs[0]
+    b = np.ascontiguousarray(a[::-1])                       # same vectors, another order
+    ctx = gpu_lib.Chi0Context(p, "fp64")
+    ctx.upload()
+
+    def call(g):
+        M = torch.zeros((2, 3, len(g)), dtype=torch.complex128, device="cuda")
+        gpu_lib.bgw_mtxel_spinor(ctx.ctx, q, g, 0, 0, 2, 0, 3, M)
+        return M
+
+    first, again, other, back = call(a), call(a), call(b), call(a)
+    torch.cuda.synchronize()
+    ctx.close()
+    assert torch.equal(first, again) and torch.equal(first, back)
+    assert torch.equal(first, other.flip(2)) and not torch.equal(first, other)
