@@ -129,7 +129,7 @@ __device__ __forceinline__ void store_kept(const C (&a)[N], C *o, int stride, in
 // ------------------------------------------------------ sphere -> grid --
 // Pass x: one thread per (band component b, y', z') line of the cube.
 template <int N>
-__global__ void __launch_bounds__(kLineThreads)
+__global__ void __launch_bounds__(kLineThreads, sizeof(T) == 8 && N <= 24 ? 3 : 0)   // 24^3 FP64: 66 -> 58 us with three CTAs per SM
 k1_xpass(const double2 *__restrict__ coeff, int ngw, long B, const int *__restrict__ cube_map,
          int w0, int w1, int w2, int s0, C *__restrict__ S) {
     const long yzs = (long)w1 * w2;
