@@ -66,6 +66,10 @@ METRIC = "spinor chi0 q-points/s and TFLOP/s, FP64 vs mixed at ≤2e-5 rel. Frob
 # i.e. 2 DFMA per clock per SM.  Peak = 152 * 2 * 2 * 2.07e9.  The roofline
 # denominator of FP64 ALU stages is the DGEMM rate measured in the same run.
 FP64_PEAK_DERIVED_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
+# FP64 transforms that run in 64-bit fixed point (square y-z planes up to 40):
+# the FP64-equivalent rate of a 24-point line, 550 flop in 2456 measured issue
+# cycles of a warp, on 4 schedulers of 152 SMs.
+FIX_PEAK_TFLOPS = 550 * 32 * 4 * 152 * 2.07e9 / 2456 / 1e12
 
 # FP32 FFMA peak from unit counts and clocks: 152 SMs x 128 lanes x 2 flop x
 # 2.07 GHz.
@@ -642,8 +646,9 @@ def measure(B, torch, p, precision, args, dist, stream, dev_in, local, with_cloc
     # achieved algorithmic rate and roofline fraction of each stage with a FLOP model
     fl = flop_model(p)
     burst, sustained, _ = bf16_peaks()
-    f64 = (args.fp64_peak, args.fp64_peak_label)
-    f64c = f64 if args.fp64_dfma else (sustained / 15, "BF16 sustained / 15 digit products")
+    f64 = ((FIX_PEAK_TFLOPS, "64-bit fixed-point line transforms (issue-bound, measured)") if fixed_grids(p) else
+           (args.fp64_peak, args.fp64_peak_label))
+    f64c = (args.fp64_peak, args.fp64_peak_label) if args.fp64_dfma else (sustained / 15, "BF16 sustained / 15 digit products")
     peaks = ({"wfn_to_grid": f64, "mtxel": f64, "mtxel_x": f64, "contraction": f64c}
              if precision == "fp64" else
              {"wfn_to_grid": (FP32_PEAK_TFLOPS, "FP32 ALU (derived)"),
@@ -685,10 +690,13 @@ def epsinv_measure(B, torch, p, res, stream, fp64_peak, reps=3):
         times.append(e0.elapsed_time(e1))
     ms = statistics.median(times[1:])
     tf = 8.0 * ng ** 3 * nf / (ms * 1e-3) / 1e12
-    return {"what": "W = eps^-1 v(q+G') for every frequency of one q (FP64, blocked Gauss-Jordan on "
-                    "the symmetrised eps)", "n_g": ng, "n_freq": nf, "ms_per_q": ms, "tflops": tf,
-            "peak_tflops": fp64_peak, "peak": "FP64 DGEMM (measured in this run)",
-            "roofline_frac": tf / fp64_peak, "derived_fp64_peak_tflops": FP64_PEAK_DERIVED_TFLOPS}
+    peak = bf16_peaks()[1] / 36
+    return {"what": "W = eps^-1 v(q+G') for every frequency of one q (FP64 accurate, blocked Gauss-Jordan on "
+                    "the symmetrised eps; panels and updates as 36 BF16 digit products on tensor cores)",
+            "n_g": ng, "n_freq": nf, "ms_per_q": ms, "tflops": tf,
+            "peak_tflops": peak, "peak": "sustained BF16 / 36 digit products (measured)",
+            "roofline_frac": tf / peak, "times_fp64_dgemm": tf / fp64_peak,
+            "derived_fp64_peak_tflops": FP64_PEAK_DERIVED_TFLOPS}
 
 
 def unfold_measure(B, torch, p, dev_in, stream, reps=3):
@@ -721,17 +729,12 @@ def unfold_measure(B, torch, p, dev_in, stream, reps=3):
     nbytes = 2 * cin.numel() * cin.element_size()
     gbs = nbytes / (ms * 1e-3) / 1e9
     hbm = measured_hbm_gbs()
-    # per band, spin pair and plane wave: the 2 x 2 complex product, 16 FP64
-    # fused multiply-adds (the phase is folded into U once per plane wave)
-    dfma = 16.0 * nb * ngw
-    dfma_peak = FP64_PEAK_DERIVED_TFLOPS * 1e12 / 2      # DFMA instructions per second
     del cin, cout
     return {"what": "c(G) -> U c(R^-1 G) e^{-iG.tau} (FP64), one launch over the bands of the step's "
                     "k-points (at most 16384) on the sphere of k-point 0",
             "bands": nb, "plane_waves": ngw, "bytes": nbytes, "ms": ms, "gbs": gbs, "peak_gbs": hbm,
             "hbm_frac": gbs / hbm if hbm else None,
-            "fp64_fma_per_s": dfma / (ms * 1e-3), "fp64_frac": dfma / (ms * 1e-3) / dfma_peak,
-            "bound": "alu (FP64): 16 DFMA per 64 bytes outruns the DRAM time on this part"}
+            "bound": "alu (integer): the 2 x 2 complex product of a spin pair runs as 48 integer multiply-adds"}
 
 
 def e2e_measure(B, torch, p, res, args, dist, stream):
@@ -927,9 +930,15 @@ def nq_of(p):
     return len(p.qs)
 
 
+def fixed_grids(p):
+    """FP64 contexts of this box keep integer grids (the library's rule)."""
+    return p.box[1] == p.box[2] <= 40
+
+
 def zy_kernel_name(p, precision, zy):
     """The kernel of the pair density + z + y stage for this box and choice
-    (the library's rule: FP64 separate passes; eight lanes per line on cubic
+    (the library's rule: FP64 separate passes, where fixed_grids does not hold;
+    eight lanes per line on cubic
     48^3/64^3; else the streamed kernel on even boxes up to 32 unless the
     plane kernel was chosen)."""
     n = p.box[1]
@@ -1017,11 +1026,13 @@ def head_roofline(p, res, precision, args, steps):
                  "unit": "TFLOP/s", "frac": ach / pk, "peak_source": lab}
     else:
         ach = fl["mtxel"] / (mt * 1e-3) / 1e12
-        pk = args.fp64_peak if precision == "fp64" else FP32_PEAK_TFLOPS
-        kern = zy_kernel_name(p, precision, (res.get("tuning") or {}).get("mtxel_zy", args.mtxel_zy))
+        fix = precision == "fp64" and fixed_grids(p)
+        pk = FIX_PEAK_TFLOPS if fix else args.fp64_peak if precision == "fp64" else FP32_PEAK_TFLOPS
+        kern = "k2_zy_fix" if fix else zy_kernel_name(p, precision, (res.get("tuning") or {}).get("mtxel_zy", args.mtxel_zy))
         r = {"bound": "alu", "kernel": kern + " (pair density + pruned z and y FFT passes)",
              "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
-             "peak_source": (args.fp64_peak_label if precision == "fp64" else
+             "peak_source": ("64-bit fixed-point line transforms (issue-bound, measured)" if fix else
+                             args.fp64_peak_label if precision == "fp64" else
                              "FP32 FFMA from unit counts: 152 SMs x 128 lanes x 2 flop x 2.07 GHz")}
     r["traffic"] = traffic
     if note:

@@ -116,7 +116,9 @@ BGW_API const char *bgw_version(void);
  *   prec    : BGW_FP64, BGW_MIXED_BF16X3, BGW_MIXED_TF32X3 or BGW_MIXED_TF32
  *   stream  : cudaStream_t to queue all work on (NULL = default stream)
  * The real-space grids, nk * (nv+nc_max) * 2 * N1*N2*N3 complex values
- * (complex128 for FP64, complex64 for mixed; fewer with BGW_OPT_GRID_SLOTS),
+ * (complex128 for FP64, complex64 for mixed; fewer with BGW_OPT_GRID_SLOTS;
+ * FP64 with fft[1] == fft[2] <= 40: 128-bit integer pairs and 4 bytes of scale
+ * per band and x-plane),
  * are allocated on the current device at the first bgw_wfn_upload.
  * Errors: BGW_E_ARG, BGW_E_NOMEM, BGW_E_CUDA.
  */
@@ -239,8 +241,9 @@ BGW_API bgw_status bgw_chi0_resume(bgw_ctx ctx, int nq, const bgw_q *qs, int nfr
  * bgw_epsinv_workspace_bytes: device workspace bgw_epsinv needs.
  * bgw_epsinv: for each of the nfreq matrices chi[j] (device, complex128
  *   [nfreq][ng][ng], row G, column G'; overwritten) forms the Hermitian
- *   eps~ = I - S chi S (S = diag(s), s on the host) and inverts it in FP64 on
- *   the GPU (blocked Gauss-Jordan without pivoting: eps~ is positive definite
+ *   eps~ = I - S chi S (S = diag(s), s on the host) and inverts it to FP64
+ *   accuracy on the GPU (blocked Gauss-Jordan without pivoting, its products on
+ *   tensor cores from BF16 digits from ng = 96 on: eps~ is positive definite
  *   when chi is Hermitian negative semidefinite, as chi0 on the imaginary axis
  *   is).  Output per mode: 0 eps~^-1; 1 W = S eps~^-1 S (eV); 2 the paper's
  *   eps^-1 = S eps~^-1 S^-1 (needs every s > 0).  work: device workspace of
@@ -248,7 +251,8 @@ BGW_API bgw_status bgw_chi0_resume(bgw_ctx ctx, int nq, const bgw_q *qs, int nfr
  *   call then allocates and frees it).  Runs on `stream` and waits for it.
  *   BGW_E_ARG for bad sizes, s < 0 or non-finite, or when a pivot is not
  *   positive (the input is not negative semidefinite; the output is then
- *   invalid); BGW_E_NOMEM / BGW_E_CUDA on allocation or CUDA failure.
+ *   invalid); BGW_E_NOMEM / BGW_E_CUDA on allocation or CUDA failure;
+ *   BGW_E_TIMEOUT if a bounded device-side wait gave up.
  *   Errors are reported by bgw_last_error(NULL).  The paper has no
  *   counterpart of the symmetrised form; it is the standard way to make the
  *   inversion Hermitian positive definite.
@@ -344,8 +348,10 @@ BGW_API bgw_status bgw_graph_launch(bgw_ctx ctx);
  *                        is cubic with N = 32, 40, 48 or 64 (else automatic),
  *                        4 (FP32 cubic boxes below 48) one kernel per band
  *                        component without the shared cube, three per SM,
- *                        where it fits (else automatic).  All give the same
- *                        grids up to rounding.
+ *                        where it fits (else automatic).  FP64 contexts with
+ *                        integer grids (see bgw_create): 0 writes them directly,
+ *                        the others build an FP64 grid and convert it.  All give
+ *                        the same grids up to rounding.
  *   BGW_OPT_MTXEL_LANES  FFT lanes per line of the matrix-element kernels:
  *                        0 automatic (default: eight for cubic 48 and 64 boxes,
  *                        one elsewhere), 1 one, 8 eight where the box is cubic
@@ -480,7 +486,8 @@ BGW_API bgw_status bgw_profile_read(bgw_ctx ctx, double *ms, long *calls, long *
  * block in an allocator.  It needs no context: the caller passes the
  * real-space grids and the output, and the call computes
  *     M[v][c][g] = N^-3 sum_r sum_alpha conj(Uv[v][alpha](r)) Uc[c][alpha](r) e^{-i(G_g+G0).r}
- * in FP64 with the same kernels as bgw_mtxel_spinor.
+ * with FP64 pair densities (the contexts' integer grids suit only grids that
+ * come from a transform) and the transforms of bgw_mtxel_spinor.
  *   fft[3] : FFT box (supported lengths as above)
  *   Uv     : DEVICE complex128 [nv][2][N1*N2*N3], u_{v,k,alpha}(r) with
  *            u(r) = sum_h c(h) e^{+2 pi i h.r/N} (unnormalised)
@@ -552,7 +559,9 @@ BGW_API bgw_status bgw_mtxel_bands(bgw_ctx ctx, const bgw_q *q, int ik, int n0, 
  *           bgw_epsinv mode 1 applied to the static chi0 of this q
  *   vq    : host [q->ng], v(q+G) in eV (the square of bgw_coulomb_sqrt)
  * Needs a BGW_FP64 context; uses context-owned scratch of about
- * 32 (nv+nc_max) nn q->ng bytes.  Waits for the stream (the sums are read
+ * 32 (nv+nc_max) nn q->ng bytes and, for ng >= 32, up to 1 GiB of digits for
+ * the products (about the same again).  BGW_E_TIMEOUT if a device-side wait of
+ * a product gave up (sx, coh unchanged).  Waits for the stream (the sums are read
  * back); not capturable (BGW_E_STATE during a capture).
  */
 BGW_API bgw_status bgw_sigma_cohsex(bgw_ctx ctx, const bgw_q *q, int ik, int n0, int nn, const void *W_dev,
@@ -578,7 +587,9 @@ BGW_API bgw_status bgw_sigma_cohsex(bgw_ctx ctx, const bgw_q *q, int ik, int n0,
  *   KX_dev, KD_dev : caller-owned DEVICE complex128 [nv*nc][nv*nc]; either
  *                 may be NULL to skip that kernel
  * Needs a BGW_FP64 context with both k-points uploaded; context-owned
- * scratch.  Asynchronous (the host v0_coul is read before the call returns).
+ * scratch, the products as in bgw_sigma_cohsex (a device-side wait that gave up
+ * shows at the next host finalize, checkpoint or bgw_sigma_cohsex).
+ * Asynchronous (the host v0_coul is read before the call returns).
  */
 BGW_API bgw_status bgw_bse_kernel(bgw_ctx ctx, int ik, int jk, const bgw_q *q0, const double *v0_coul,
                                   const bgw_q *qd, const void *W_dev, int v0, int nv, int c0, int nc,
