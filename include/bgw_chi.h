@@ -117,7 +117,7 @@ BGW_API const char *bgw_version(void);
  *   stream  : cudaStream_t to queue all work on (NULL = default stream)
  * The real-space grids, nk * (nv+nc_max) * 2 * N1*N2*N3 complex values
  * (complex128 for FP64, complex64 for mixed; fewer with BGW_OPT_GRID_SLOTS;
- * FP64 with fft[1] == fft[2] <= 40: 128-bit integer pairs and 4 bytes of scale
+ * FP64 with fft[1] == fft[2] <= 40: 128-bit integer pairs and 8 bytes of scales
  * per band and x-plane),
  * are allocated on the current device at the first bgw_wfn_upload.
  * Errors: BGW_E_ARG, BGW_E_NOMEM, BGW_E_CUDA.

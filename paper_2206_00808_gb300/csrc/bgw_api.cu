@@ -278,11 +278,11 @@ struct bgw_ctx_s {
     }
     long grid_elems_per_k() const { return (long)nb * 2 * nbox; }
     // FP64 contexts whose grids are integer grids (bgw_internal.h): the scales
-    // [slot][band][N1] follow the grids in the same allocation
+    // [slot][band][2][N1] follow the grids in the same allocation
     bool fixed = false;
     int *scale_ptr(int slot, int band) {
         return reinterpret_cast<int *>(static_cast<char *>(grids.p) + (size_t)nslots * grid_elems_per_k() * csize) +
-               ((long)slot * nb + band) * box[0];
+               ((long)slot * nb + band) * 2 * box[0];
     }
     char *slot_ptr(int slot, int band) {
         return static_cast<char *>(grids.p) + ((long)slot * grid_elems_per_k() + (long)band * 2 * nbox) * csize;
@@ -308,7 +308,7 @@ cudaError_t ensure_slots(bgw_ctx_s *c) {
     if (c->nslots > 0) return cudaSuccess;
     const int n = (c->grid_slots_opt > 0 && c->grid_slots_opt < c->nk) ? std::max(2, c->grid_slots_opt)
                                                                          : c->nk;
-    const size_t scales = c->fixed ? sizeof(int) * (size_t)n * c->nb * c->box[0] : 0;
+    const size_t scales = c->fixed ? sizeof(int) * (size_t)n * c->nb * 2 * c->box[0] : 0;
     cudaError_t e = c->grids.ensure((size_t)n * c->grid_elems_per_k() * c->csize + scales, c->st);
     if (e != cudaSuccess) return e;
     c->nslots = n;

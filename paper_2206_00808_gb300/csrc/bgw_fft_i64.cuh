@@ -291,11 +291,16 @@ __device__ __forceinline__ void fft_line_fix(cpx<double> (&a)[N]) {
 
 // ------------------------------------------------------- integer grids --
 // Real-space grids of the FP64 contexts whose y-z planes are square and at
-// most 40 wide are kept as integers of one scale per (band, x-plane), both
-// spin components together: {re hi, re lo, im hi, im lo} with
-// u = (hi 2^32 + lo) 2^scale, |u| 2^-scale <= 2^fix_grid_top(N).  16 bytes a
-// value, as in FP64; the largest component of a plane keeps 60 bits.
+// most 40 wide are kept as integers of one scale per (band, spin component,
+// x-plane): {re hi, re lo, im hi, im lo} with u = (hi 2^32 + lo) 2^scale,
+// |u| 2^-scale <= 2^fix_grid_top(N).  16 bytes a value, as in FP64; the largest
+// component of a plane keeps 60 bits.  The two spin components of a plane share
+// the larger's scale unless one is more than 2^kFixApart smaller (a nearly
+// spin-pure state, whose small component then keeps its own 60 bits).
 constexpr int kFixBad = 1 << 24;      // scale of a plane with an infinity or a NaN
+constexpr int kFixApart = 4;
+// The scale a component with own scale s takes beside one with scale t.
+__device__ __forceinline__ int fix_shared_scale(int s, int t) { return s < t && t - s <= kFixApart ? t : s; }
 // Pair densities of two such planes stay below 2^fix_top(N).
 __host__ __device__ constexpr int fix_grid_top(int n) { return fix_top(n) >= 58 ? 60 : 59; }
 
@@ -313,6 +318,7 @@ __device__ __forceinline__ int fix_mag(i64c v) {
     const int x = (int)(v.x >> 32), y = (int)(v.y >> 32);
     return (x ^ (x >> 31)) | (y ^ (y >> 31));
 }
+// r in 1..63
 __device__ __forceinline__ long long fix_shift_right(long long v, int r) { return (v + (1LL << (r - 1))) >> r; }
 
 }  // namespace bgw

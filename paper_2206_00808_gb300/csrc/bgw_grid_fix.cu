@@ -38,7 +38,7 @@ k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
     constexpr int XP = K1Tile<N>::XP, THREADS = K1Tile<N>::THREADS, RS = K1Tile<N>::RS;
     constexpr int NN = N * N, TOP = fix_top(N), GTOP = fix_grid_top(N);
     extern __shared__ int4 yz_raw[];
-    __shared__ int smax[XP], ybits[XP], zbits[XP];
+    __shared__ int smax[2 * XP], ybits[2 * XP], zbits[2 * XP];      // per (spin component, plane)
     const int x0 = blockIdx.x * XP, xp = min(XP, n0 - x0);
     const long b = blockIdx.y;
     const int cells = w1 * w2, w2p = w2 | 1;
@@ -46,7 +46,7 @@ k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
     // z outputs, over both
     i64c *A = reinterpret_cast<i64c *>(yz_raw), *Y = A + 2 * XP * cells;
     int4 *Cc = yz_raw;
-    if (threadIdx.x < XP) smax[threadIdx.x] = ybits[threadIdx.x] = zbits[threadIdx.x] = 0;
+    if (threadIdx.x < 2 * XP) smax[threadIdx.x] = ybits[threadIdx.x] = zbits[threadIdx.x] = 0;
     __syncthreads();
     double2 *Ad = reinterpret_cast<double2 *>(yz_raw);
     for (int al = 0; al < 2; ++al)
@@ -60,12 +60,12 @@ k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
                 m = max(m, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
             }
             m = __reduce_max_sync(0xffffffffu, m);
-            if ((threadIdx.x & 31) == 0) atomicMax(&smax[xl], m);
+            if ((threadIdx.x & 31) == 0) atomicMax(&smax[al * XP + xl], m);
         }
     __syncthreads();
     for (int al = 0; al < 2; ++al)
         for (int xl = 0; xl < xp; ++xl) {
-            const int E = smax[xl] >> 20;
+            const int E = smax[al * XP + xl] >> 20;
             double2 *a = Ad + (al * XP + xl) * cells;
             for (int i = threadIdx.x; i < cells; i += THREADS) {       // each thread its own values
                 const double2 v = a[i];
@@ -92,12 +92,12 @@ k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
             o[y * w2p] = a[y];
             big |= fix_mag(a[y]);
         }
-        atomicMax(&ybits[xl], 64 - __clz(big));
+        atomicMax(&ybits[q], 64 - __clz(big));
     }
     __syncthreads();
     const int q = threadIdx.x / N, y = threadIdx.x % N, xl = q % XP;
     const bool line = q < 2 * XP && xl < xp;
-    const int r = line ? max(0, ybits[xl] - TOP) : 0;
+    const int r = line ? max(0, ybits[q] - TOP) : 0;
     i64c a[N];
     if (line) {
         const i64c *row = Y + (q * N + y) * w2p;
@@ -114,11 +114,16 @@ k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
         int big = 0;
 #pragma unroll
         for (int z = 0; z < N; ++z) big |= fix_mag(a[z]);
-        atomicMax(&zbits[xl], 64 - __clz(big));
+        atomicMax(&zbits[q], 64 - __clz(big));
     }
     __syncthreads();                       // Y has been read: the outputs go over it
     if (line) {
-        const int sh = GTOP - zbits[xl];
+        // the exponent of this plane's integers, the scale that brings its largest
+        // value to GTOP bits, and the same for the other spin component
+        auto raw = [&](int i) { return (smax[i] >> 20) - 1022 - TOP + 2 * fix_levels(N) + max(0, ybits[i] - TOP); };
+        const int other = q < XP ? q + XP : q - XP;
+        const int s = fix_shared_scale(raw(q) + zbits[q] - GTOP, raw(other) + zbits[other] - GTOP);
+        const int sh = max(raw(q) - s, -63);
         int4 *o = Cc + (q * N + y) * RS;
         if (sh >= 0) {
 #pragma unroll
@@ -127,10 +132,7 @@ k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
 #pragma unroll
             for (int z = 0; z < N; ++z) o[z] = fix_pack(fix_shift_right(a[z].x, -sh), fix_shift_right(a[z].y, -sh));
         }
-        if (y == 0 && q < XP) {
-            const int E = smax[xl] >> 20;
-            scale[b * n0 + x0 + xl] = E == 0x7ff ? kFixBad : E - 1022 - TOP + 2 * fix_levels(N) + r - sh;
-        }
+        if (y == 0) scale[(2 * b + q / XP) * n0 + x0 + xl] = smax[q] >> 20 == 0x7ff ? kFixBad : s;
     }
     __syncthreads();
     for (int al = 0; al < 2; ++al) {
@@ -147,29 +149,38 @@ k_fix_planes(void *__restrict__ U, int *__restrict__ scale) {
     constexpr int NN = N * N, IT = (2 * NN + kConvThreads - 1) / kConvThreads, TOP = fix_grid_top(N);
     const int x = blockIdx.x, n0 = gridDim.x;
     const long b = blockIdx.y;
-    __shared__ int smax;
-    if (threadIdx.x == 0) smax = 0;
+    __shared__ int smax[2];
+    if (threadIdx.x < 2) smax[threadIdx.x] = 0;
     double2 v[IT];
-    int m = 0;
+    int m[2] = {0, 0};
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
         const int t = i * kConvThreads + threadIdx.x;
         v[i] = make_double2(0.0, 0.0);
         if (t < 2 * NN) v[i] = static_cast<double2 *>(U)[((2 * b + t / NN) * n0 + x) * NN + t % NN];
-        m = max(m, max(__double2hiint(v[i].x) & 0x7fffffff, __double2hiint(v[i].y) & 0x7fffffff));
+        const int mi = max(__double2hiint(v[i].x) & 0x7fffffff, __double2hiint(v[i].y) & 0x7fffffff);
+        m[0] = max(m[0], t < NN ? mi : 0);
+        m[1] = max(m[1], t < NN ? 0 : mi);
     }
     __syncthreads();
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(&smax, m);
+#pragma unroll
+    for (int al = 0; al < 2; ++al) {
+        m[al] = __reduce_max_sync(0xffffffffu, m[al]);
+        if ((threadIdx.x & 31) == 0) atomicMax(&smax[al], m[al]);
+    }
     __syncthreads();
-    const int E = smax >> 20;
-    if (threadIdx.x == 0) scale[b * n0 + x] = E == 0x7ff ? kFixBad : E - 1022 - TOP;
+    const int E0 = smax[0] >> 20, E1 = smax[1] >> 20;
+    const int e0 = fix_shared_scale(E0, E1), e1 = fix_shared_scale(E1, E0);
+    if (threadIdx.x < 2) {
+        const int E = threadIdx.x ? E1 : E0, e = threadIdx.x ? e1 : e0;
+        scale[(2 * b + threadIdx.x) * n0 + x] = E == 0x7ff ? kFixBad : e - 1022 - TOP;
+    }
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
         const int t = i * kConvThreads + threadIdx.x;
         if (t < 2 * NN)
             static_cast<int4 *>(U)[((2 * b + t / NN) * n0 + x) * NN + t % NN] =
-                fix_pack(fix_in<TOP>(v[i].x, E), fix_in<TOP>(v[i].y, E));
+                fix_pack(fix_in<TOP>(v[i].x, t < NN ? e0 : e1), fix_in<TOP>(v[i].y, t < NN ? e0 : e1));
     }
 }
 
@@ -178,10 +189,11 @@ __global__ void __launch_bounds__(kConvThreads)
 k_unfix_planes(const int4 *__restrict__ F, const int *__restrict__ scale, int n0, int NN, double2 *__restrict__ U) {
     const int x = blockIdx.x;
     const long b = blockIdx.y;
-    const int s = scale[b * n0 + x];
+    const int s0 = scale[2 * b * n0 + x], s1 = scale[(2 * b + 1) * n0 + x];
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     for (int t = threadIdx.x; t < 2 * NN; t += kConvThreads) {
         const long at = ((2 * b + t / NN) * n0 + x) * NN + t % NN;
+        const int s = t < NN ? s0 : s1;
         const int4 f = F[at];
         double2 v = make_double2(fix_out(fix_unpack(f.x, f.y), 1086 + s), fix_out(fix_unpack(f.z, f.w), 1086 + s));
         if (s == kFixBad) v = make_double2(nan, nan);

@@ -1739,7 +1739,7 @@ static cudaError_t mtxel(const void *Uv, const void *Uc, int nv, int nc, const A
         const int nvb = nv - vb0 < VB ? nv - vb0 : VB;
         cudaError_t e = mtxel_batch(uv + (long)vb0 * 2 * vol, uc, nvb, nc, a, gmap, ng, Ap, Bp,
                                     Mp + (long)vb0 * nc * ldm, ldm, st, tv_req, tc_req, lanes, zy, hook, err, drop,
-                                    sv ? sv + (long)vb0 * a.n[0] : nullptr, sc);
+                                    sv ? sv + 2L * vb0 * a.n[0] : nullptr, sc);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

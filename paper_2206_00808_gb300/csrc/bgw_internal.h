@@ -157,7 +157,7 @@ cudaError_t zy_fix_tables_init();
 cudaError_t wfn_xpass_f64(const double *coeff, int ngw, int B, const int *cube_map, const Axes &a, void *S,
                           cudaStream_t st);
 // wfn_to_grid for nb bands into an integer grid: U [nb][2][N^3] of 16 bytes,
-// scale [nb][n0].
+// scale [nb][2][n0].
 cudaError_t wfn_to_fix(const double *coeff, int ngw, int nb, const int *cube_map, const Axes &a, void *S, void *U,
                        int *scale, cudaStream_t st);
 // FP64 grid to integer grid in place, and an integer grid to an FP64 one.

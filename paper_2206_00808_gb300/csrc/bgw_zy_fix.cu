@@ -50,10 +50,18 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
     extern __shared__ int4 zy_raw[];
     i64c *R = reinterpret_cast<i64c *>(zy_raw);      // [TV*TC][N][RS]
     __shared__ int pbits[TV * TC];
+    __shared__ int apart[TV * TC];     // exponent of the spin-up products over the spin-down ones
     const int x = blockIdx.x, n0 = gridDim.x;
     const int v0 = blockIdx.y * TV, c0 = blockIdx.z * TC;
     const int tv = min(TV, nv - v0), tc = min(TC, nc - c0);
-    if (threadIdx.x < TV * TC) pbits[threadIdx.x] = 0;
+    const auto scale_v = [&](int v, int al) { return Sv[(2L * (v0 + v) + al) * n0 + x]; };
+    const auto scale_c = [&](int c, int al) { return Sc[(2L * (c0 + c) + al) * n0 + x]; };
+    if (threadIdx.x < TV * TC) {
+        const int v = min((int)threadIdx.x / TC, tv - 1), c = min((int)threadIdx.x % TC, tc - 1);
+        pbits[threadIdx.x] = 0;
+        apart[threadIdx.x] = scale_v(v, 0) + scale_c(c, 0) - scale_v(v, 1) - scale_c(c, 1);
+    }
+    __syncthreads();
     // 1. pair densities (a tile's missing bands repeat its last one)
     const int4 *pv[TV], *pc[TC];
 #pragma unroll
@@ -76,6 +84,22 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
 #pragma unroll
             for (int i = 0; i < TC; ++i) {
                 const int4 p = c[i][0], q = c[i][1];
+                const int ap = apart[v * TC + i];
+                if (ap != 0) {        // the spin components have scales of their own: join each, align the smaller
+                    auto part = [&](const int4 &a4, int nh, int nl, const int4 &p4) {
+                        const long long rh = fix_mad(a4.x, p4.x, fix_mad(a4.z, p4.z, 0));
+                        const long long rl = fix_mad(a4.x, p4.y, fix_mad(a4.y, p4.x, fix_mad(a4.z, p4.w, fix_mad(a4.w, p4.z, kFixHalf))));
+                        const long long ih = fix_mad(a4.x, p4.z, fix_mad(nh, p4.x, 0));
+                        const long long il = fix_mad(a4.x, p4.w, fix_mad(a4.y, p4.z, fix_mad(nh, p4.y, fix_mad(nl, p4.x, kFixHalf))));
+                        return i64c{fix_join(rh, rl), fix_join(ih, il)};
+                    };
+                    i64c up = part(a, nah, nal, p), dn = part(b, nbh, nbl, q);
+                    const int r1 = min(ap < 0 ? -ap : ap, 63);
+                    if (ap < 0) up = i64c{fix_shift_right(up.x, r1), fix_shift_right(up.y, r1)};
+                    else dn = i64c{fix_shift_right(dn.x, r1), fix_shift_right(dn.y, r1)};
+                    r[(v * TC + i) * N * RS] = cadd(up, dn);
+                    continue;
+                }
                 const long long reh = fix_mad(a.x, p.x, fix_mad(a.z, p.z, fix_mad(b.x, q.x, fix_mad(b.z, q.z, 0))));
                 long long rel = fix_mad(a.x, p.y, fix_mad(a.y, p.x, fix_mad(a.z, p.w, fix_mad(a.w, p.z, kFixHalf))));
                 rel = fix_mad(b.x, q.y, fix_mad(b.y, q.x, fix_mad(b.z, q.w, fix_mad(b.w, q.z, rel))));
@@ -127,9 +151,9 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
             for (int y = 0; y < N; ++y) a[y] = i64c{fix_shift_right(a[y].x, r), fix_shift_right(a[y].y, r)};
         }
         FixFft<-1, N, N>::run(a);
-        const int ev = Sv[(long)(v0 + v) * n0 + x], ec = Sc[(long)(c0 + c) * n0 + x];
-        const bool bad = ev == kFixBad || ec == kFixBad;
-        const int eb = 1086 + ev + ec + 64 + 2 * fix_levels(N) + r;
+        const int v0s = scale_v(v, 0), v1s = scale_v(v, 1), c0s = scale_c(c, 0), c1s = scale_c(c, 1);
+        const bool bad = v0s == kFixBad || v1s == kFixBad || c0s == kFixBad || c1s == kFixBad;
+        const int eb = 1086 + max(v0s + c0s, v1s + c1s) + 64 + 2 * fix_levels(N) + r;
         const double nan = __longlong_as_double(0x7ff8000000000000ll);
         double2 *o = Bs + (((long)(v0 + v) * ldc + c0 + c) * n0 + x) * w1 * (long)w2 + jz;
         constexpr int K = WIN ? 2 * kWinF + 1 : N;

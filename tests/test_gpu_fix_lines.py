@@ -72,3 +72,16 @@ def test_scales_and_non_finite_bands(gpu_lib):
     assert (got[2, :4] == 0).all()
     for v in (1, 3):
         assert (got[v, :4] == base[v, :4] * scale[v, :4, None]).all()
+
+
+def test_small_spin_components_keep_their_precision(gpu_lib):
+    """A nearly spin-up valence band against spin-down conduction bands: the
+    element comes from the small components alone and is as exact as any."""
+    torch = pytest.importorskip("torch")
+    p = syn.make_problem("si18_qx", nv=3, nc=4)
+    for c in p.coeff:
+        c[:p.nv, 1] *= 2.0 ** -40                # valence: spin down 1e-12 of spin up
+        c[p.nv:, 0] = 0.0                        # conduction: spin down only
+        c[p.nv + 1, 0] = c[p.nv + 1, 1] * 2.0 ** -50
+    got, ref = mtxel(gpu_lib, torch, p, 4, 0, 3, 0, 4), reference(p, 4, 0, 3, 0, 4)
+    assert np.abs(got - ref).max() <= TOL * np.abs(ref).max()
