@@ -17,6 +17,8 @@
 // the FP64 pipe, whose operations cost 64 to 76 such cycles.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "bgw_fft_i64.cuh"
 #include "bgw_internal.h"
 
@@ -56,12 +58,14 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
     const int tv = min(TV, nv - v0), tc = min(TC, nc - c0);
     const auto scale_v = [&](int v, int al) { return Sv[(2L * (v0 + v) + al) * n0 + x]; };
     const auto scale_c = [&](int c, int al) { return Sc[(2L * (c0 + c) + al) * n0 + x]; };
+    int ap = 0;
     if (threadIdx.x < TV * TC) {
         const int v = min((int)threadIdx.x / TC, tv - 1), c = min((int)threadIdx.x % TC, tc - 1);
         pbits[threadIdx.x] = 0;
-        apart[threadIdx.x] = scale_v(v, 0) + scale_c(c, 0) - scale_v(v, 1) - scale_c(c, 1);
+        ap = scale_v(v, 0) + scale_c(c, 0) - scale_v(v, 1) - scale_c(c, 1);
+        apart[threadIdx.x] = ap;
     }
-    __syncthreads();
+    const bool any_apart = __syncthreads_or(ap != 0);
     // 1. pair densities (a tile's missing bands repeat its last one)
     const int4 *pv[TV], *pc[TC];
 #pragma unroll
@@ -69,6 +73,9 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
 #pragma unroll
     for (int c = 0; c < TC; ++c) pc[c] = Fc + (2L * (c0 + min(c, tc - 1)) * n0 + x) * NN;
     const long spin = (long)n0 * NN;
+    // in a loop of its own where a pair's spin components have scales apart (one
+    // loop for both took 13 % longer at 32^3)
+    auto densities = [&](auto slow) {
     for (int t = threadIdx.x; t < NN; t += THREADS) {
         int4 c[TC][2];
 #pragma unroll
@@ -84,8 +91,8 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
 #pragma unroll
             for (int i = 0; i < TC; ++i) {
                 const int4 p = c[i][0], q = c[i][1];
-                const int ap = apart[v * TC + i];
-                if (ap != 0) {        // the spin components have scales of their own: join each, align the smaller
+                // (pair by pair, so that a pair's bits do not depend on its tile)
+                if (decltype(slow)::value && apart[v * TC + i] != 0) {        // the spin components have scales of their own: join each, align the smaller
                     auto part = [&](const int4 &a4, int nh, int nl, const int4 &p4) {
                         const long long rh = fix_mad(a4.x, p4.x, fix_mad(a4.z, p4.z, 0));
                         const long long rl = fix_mad(a4.x, p4.y, fix_mad(a4.y, p4.x, fix_mad(a4.z, p4.w, fix_mad(a4.w, p4.z, kFixHalf))));
@@ -94,8 +101,8 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
                         return i64c{fix_join(rh, rl), fix_join(ih, il)};
                     };
                     i64c up = part(a, nah, nal, p), dn = part(b, nbh, nbl, q);
-                    const int r1 = min(ap < 0 ? -ap : ap, 63);
-                    if (ap < 0) up = i64c{fix_shift_right(up.x, r1), fix_shift_right(up.y, r1)};
+                    const int d = apart[v * TC + i], r1 = min(d < 0 ? -d : d, 63);
+                    if (d < 0) up = i64c{fix_shift_right(up.x, r1), fix_shift_right(up.y, r1)};
                     else dn = i64c{fix_shift_right(dn.x, r1), fix_shift_right(dn.y, r1)};
                     r[(v * TC + i) * N * RS] = cadd(up, dn);
                     continue;
@@ -110,6 +117,11 @@ k2_zy_fix(const int4 *__restrict__ Fv, const int *__restrict__ Sv, const int4 *_
             }
         }
     }
+    };
+    if (any_apart)
+        densities(std::true_type());
+    else
+        densities(std::false_type());
     __syncthreads();
     // 2. z lines
     const int ns1 = N - s1, ns2 = N - s2;
