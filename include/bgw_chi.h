@@ -430,7 +430,9 @@ BGW_API bgw_status bgw_graph_launch(bgw_ctx ctx);
  *                        variable BGW_FAULT=oom@n, read by bgw_create, does the
  *                        same.
  *   BGW_OPT_TEST_DROP_LOAD  for failure-handling tests only: 1, the next mixed
- *                        contractions lose one operand load on purpose, so the
+ *                        contractions (in FP64 contexts the products of
+ *                        bgw_sigma_cohsex and bgw_bse_kernel, reported by those
+ *                        calls) lose one operand load on purpose, so the
  *                        kernel's bounded waits (about 2 s) expire, it frees its
  *                        resources and records an error that a host finalize
  *                        reports as BGW_E_TIMEOUT; 2, the same for the streamed
@@ -587,9 +589,10 @@ BGW_API bgw_status bgw_sigma_cohsex(bgw_ctx ctx, const bgw_q *q, int ik, int n0,
  *   KX_dev, KD_dev : caller-owned DEVICE complex128 [nv*nc][nv*nc]; either
  *                 may be NULL to skip that kernel
  * Needs a BGW_FP64 context with both k-points uploaded; context-owned
- * scratch, the products as in bgw_sigma_cohsex (a device-side wait that gave up
- * shows at the next host finalize, checkpoint or bgw_sigma_cohsex).
- * Asynchronous (the host v0_coul is read before the call returns).
+ * scratch, the products as in bgw_sigma_cohsex.  BGW_E_TIMEOUT if a device-side
+ * wait of K^X gave up (K^D is then not formed).  Asynchronous (the host v0_coul is
+ * read and K^X complete before the call returns); where a wait of K^D gave up,
+ * the entries of KD_dev that it touches are NaN.
  */
 BGW_API bgw_status bgw_bse_kernel(bgw_ctx ctx, int ik, int jk, const bgw_q *q0, const double *v0_coul,
                                   const bgw_q *qd, const void *W_dev, int v0, int nv, int c0, int nc,

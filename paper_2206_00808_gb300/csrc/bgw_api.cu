@@ -171,7 +171,9 @@ struct bgw_ctx_s {
     DevBuf gmap_tmp;     // dielectric-sphere map of a bgw_mtxel_spinor call
     std::vector<int> gmap_host;      // its contents, while every write of it is known (see put_gmap)
     bool gmap_captured = false;
-    DevBuf errflag;      // device int: non-zero after a bounded device wait gave up
+    DevBuf errflag;      // device ints, non-zero after a bounded device wait gave up: [0] of the chi0 and
+                         // matrix-element kernels, [1] of a digit product (see dz_err)
+    int *dz_err() { return static_cast<int *>(errflag.p) + 1; }
     // scratch of the self-energy and BSE kernel calls (matrix-element blocks,
     // products, per-pair sums, a copy of the interaction's diagonal)
     DevBuf nx_m1, nx_m2, nx_y, nx_t, nx_s, nx_v, nx_dz;
@@ -1011,7 +1013,7 @@ cudaError_t row_product(bgw_ctx_s *c, long M, int N, int K, const void *A, long 
             e = bgw::dz_split(op, pl, 2, K, c->st);
             const bgw::DzOut out = {static_cast<double2 *>(C) + m0 * sc + n0, 0, sc, 1, 0, 0, alpha, 0.0, false};
             if (e == cudaSuccess)
-                e = bgw::dz_gemm(pl[0], pl[1], out, c->sm_count, c->st, static_cast<int *>(c->errflag.p));
+                e = bgw::dz_gemm(pl[0], pl[1], out, c->sm_count, c->st, c->dz_err(), c->test_drop_load == 1);
         }
     return e;
 }
@@ -1153,8 +1155,8 @@ bgw_status bgw_create(bgw_ctx *out, const int fft[3], int nk, const double *kcry
         c->sm_count = 1;
     c->k.resize(nk);
     e = c->energy.ensure(sizeof(double) * (size_t)nk * c->nb, c->st);
-    if (e == cudaSuccess) e = c->errflag.ensure(sizeof(int), c->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->errflag.p, 0, sizeof(int), c->st);
+    if (e == cudaSuccess) e = c->errflag.ensure(2 * sizeof(int), c->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->errflag.p, 0, 2 * sizeof(int), c->st);
     if (e != cudaSuccess) {
         g_create_error = std::string("bgw_create: allocating buffers: ") + cudaGetErrorString(e);
         const bgw_status s = (e == cudaErrorMemoryAllocation) ? BGW_E_NOMEM : BGW_E_CUDA;
@@ -1983,6 +1985,7 @@ bgw_status bgw_sigma_cohsex(bgw_ctx c, const bgw_q *q, int ik, int n0, int nn, c
     if (st != BGW_OK) return st;
     double *sw = static_cast<double *>(c->nx_s.p), *tv = sw + P, *out = tv + P;
     e = cudaMemcpyAsync(c->nx_v.p, vq, sizeof(double) * s.ng, cudaMemcpyHostToDevice, c->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->dz_err(), 0, sizeof(int), c->st);
     // Y[p][G] = sum_G' W[G][G'] M[p][G']
     if (e == cudaSuccess)
         e = row_product(c, P, s.ng, s.ng, c->nx_m1.p, s.ng, false, W_dev, s.ng, false, nullptr, c->nx_y.p, s.ng, 1.0);
@@ -1995,13 +1998,11 @@ bgw_status bgw_sigma_cohsex(bgw_ctx c, const bgw_q *q, int ik, int n0, int nn, c
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h.data(), out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->st);
     int flag = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c->dz_err(), sizeof(int), cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     if (e != cudaSuccess) return c->cuda_fail(e, "sigma_cohsex: kernels");
-    if (flag && flag != bgw::F64TC_ERR_SIGN) {        // a bounded wait of the product gave up: sx, coh unchanged
-        cudaMemsetAsync(c->errflag.p, 0, sizeof(int), c->st);
+    if (flag)        // a bounded wait of the product gave up: sx, coh unchanged
         return c->fail(BGW_E_TIMEOUT, "sigma_cohsex: a device-side wait gave up (code %d)", flag);
-    }
     const double scale = 1.0 / c->nk;
     for (int n = 0; n < nn; ++n) {
         sx[n] += -scale * h[n];
@@ -2046,12 +2047,16 @@ bgw_status bgw_bse_kernel(bgw_ctx c, int ik, int jk, const bgw_q *q0, const doub
         if (st == BGW_OK) st = mtxel_into(c, "bse_kernel", s, jk, va, nv, ca, nc, c->nx_m2.p, clean);
         if (st != BGW_OK) return st;
         e = cudaMemcpyAsync(c->nx_v.p, v0_coul, sizeof(double) * s.ng, cudaMemcpyHostToDevice, c->st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->dz_err(), 0, sizeof(int), c->st);
         // KX[I][J] = (1/N_k) sum_G v(G) M_I(k_i, G) conj(M_J(k_j, G))
         if (e == cudaSuccess)
             e = row_product(c, P, (int)P, s.ng, c->nx_m1.p, s.ng, false, c->nx_m2.p, s.ng, true,
                             static_cast<const double *>(c->nx_v.p), KX_dev, P, scale);
+        int flag = 0;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c->dz_err(), sizeof(int), cudaMemcpyDeviceToHost, c->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);   // the host copy of v(G) has been read
         if (e != cudaSuccess) return c->cuda_fail(e, "bse_kernel: exchange");
+        if (flag) return c->fail(BGW_E_TIMEOUT, "bse_kernel: a device-side wait of K^X gave up (code %d)", flag);
     }
     if (KD_dev) {
         QState s;

@@ -26,7 +26,8 @@
 //           warp 17 MMA (72 of M128 N64 K16 a block), warps 0-15 promote and
 //           write.  Bound: shared-memory reads of the MMAs (a 128 x 64 x 16 MMA
 //           reads 6 KB, 48 clocks, against 32 of the tensor core).
-// Every mbarrier wait is bounded, as in bgw_chi0_f64tc.cu.
+// Every mbarrier wait is bounded, as in bgw_chi0_f64tc.cu; a block whose wait gave
+// up writes NaN for the rest of its tiles, so that what is built on them shows it.
 #include "bgw_dz.h"
 
 #include <cuda.h>
@@ -240,6 +241,7 @@ struct GemmArgs {
     int b0a, b0b;            // first matrix of each operand's planes
     int nkb, items;
     int alpha;               // kOne ...: no FP64 compare per output
+    int drop;                // test hook: block 0 never issues its first stage
 };
 
 __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__ GemmArgs g, int *__restrict__ err) {
@@ -273,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
 
     if (warp == kEpi) {
         if (lane == 0) {
-            long pit = 0;
+            long pit = 0, dropped = -1;
             bool stop = false;
             for (int item = blockIdx.x; item < g.items && !stop; item += gridDim.x) {
                 const int b = item / per, ti = item % per / g.tb, tj = item % per % g.tb;
@@ -290,6 +292,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                         stop = true;
                         break;
                     }
+                    if (g.drop && blockIdx.x == 0 && pit == 0) {
+                        dropped = pit;
+                        continue;
+                    }
                     const uint32_t st0 = ring + s * kStage, fb = smem_u32(&full_bar[s]);
                     mbar_expect_tx(fb, kStage);
                     for (int t = 0; t < kSl; ++t) {
@@ -301,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
             }
             // every issued load must land before the CTA can exit
             for (long q = pit > kStg ? pit - kStg : 0; q < pit; ++q)
-                if (!mbar_wait(smem_u32(&full_bar[q % kStg]), (uint32_t)((q / kStg) & 1))) {
+                if (q != dropped && !mbar_wait(smem_u32(&full_bar[q % kStg]), (uint32_t)((q / kStg) & 1))) {
                     atomicExch(err, kErrDrain);
                     break;
                 }
@@ -362,6 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
         const int quarter = warp & 3, group = warp >> 2;
         const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(16 * group);
         long gsub = 0;
+        bool ok = true;
         for (int item = blockIdx.x; item < g.items; item += gridDim.x) {
             const int b = item / per, ti = item % per / g.tb, tj = item % per % g.tb;
             long long n[16];       // sum of orders 0-5 in units of 2^-36,
@@ -372,12 +379,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                 f[i] = 0.f;
             }
             const int nsub = (g.nkb + kSub - 1) / kSub;
-            bool ok = true;
-            for (int sub = 0; sub < nsub; ++sub, ++gsub) {
+            for (int sub = 0; sub < nsub && ok; ++sub, ++gsub) {
                 bool got = mbar_wait(smem_u32(&set_full), (uint32_t)(gsub & 1));
                 got = __all_sync(0xffffffffu, got && !*(volatile int *)&abort_flag);
-                if (!got) {
+                if (!got) {                     // no further waits: NaN for this tile and the rest
                     if (lane == 0) atomicExch(err, kErrAccum);
+                    atomicExch(&abort_flag, 1);
                     ok = false;
                     break;
                 }
@@ -414,10 +421,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 mbar_arrive(smem_u32(&set_free));
             }
-            if (!ok) {
-                atomicExch(&abort_flag, 1);
-                break;
-            }
             const int m = ti * kM + 32 * quarter + lane;
             const int n0 = (tj * kN + 16 * group) / 2;
             const DzOut &o = g.out;
@@ -446,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                         d[h] = fix_out(x, 1086 - 36 - sh + ea + eb);
                     }
                     double2 r = make_double2(d[0], d[1]);
-                    if (ea == kFixBad || eb == kFixBad) r.x = r.y = __longlong_as_double(0x7ff8000000000000ll);
+                    if (ea == kFixBad || eb == kFixBad || !ok) r.x = r.y = __longlong_as_double(0x7ff8000000000000ll);
                     if (g.alpha == kComplex)
                         r = make_double2(o.ar * r.x - o.ai * r.y, o.ar * r.y + o.ai * r.x);
                     else if (g.alpha == kReal)
@@ -522,7 +525,8 @@ cudaError_t dz_split(const DzOperand *op, const DzPlanes *pl, int n, int K, cuda
     return cudaGetLastError();
 }
 
-cudaError_t dz_gemm(const DzPlanes &A, const DzPlanes &B, const DzOut &out, int sm_count, cudaStream_t st, int *err) {
+cudaError_t dz_gemm(const DzPlanes &A, const DzPlanes &B, const DzOut &out, int sm_count, cudaStream_t st, int *err,
+                    bool drop) {
     GemmArgs g;
     memset(&g, 0, sizeof g);
     cudaError_t e = make_map(A, &g.ma);
@@ -542,6 +546,7 @@ cudaError_t dz_gemm(const DzPlanes &A, const DzPlanes &B, const DzOut &out, int 
     g.b0b = B.first;
     g.items = A.used * g.ta * g.tb;
     g.alpha = out.ai != 0.0 ? kComplex : out.ar == 1.0 ? kOne : out.ar == -1.0 ? kMinusOne : kReal;
+    g.drop = drop;
     const int smem = kStg * kStage + 1024;
     e = cudaFuncSetAttribute(k_dz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

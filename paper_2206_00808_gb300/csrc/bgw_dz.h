@@ -43,7 +43,10 @@ size_t dz_planes_bytes(int rows, int K, int batch, bool b);
 DzPlanes dz_planes(void *ws, int rows, int K, int batch, bool b);
 // Cut n operands into their digits, one launch (all of the same K).
 cudaError_t dz_split(const DzOperand *op, const DzPlanes *pl, int n, int K, cudaStream_t st);
-// err: device int, set non-zero when a bounded device wait gave up.
-cudaError_t dz_gemm(const DzPlanes &A, const DzPlanes &B, const DzOut &out, int sm_count, cudaStream_t st, int *err);
+// err: device int, set non-zero when a bounded device wait gave up (the outputs
+// that the block had still to write are then NaN).  drop: test hook, block 0
+// never issues its first loads.
+cudaError_t dz_gemm(const DzPlanes &A, const DzPlanes &B, const DzOut &out, int sm_count, cudaStream_t st, int *err,
+                    bool drop = false);
 
 }  // namespace bgw
