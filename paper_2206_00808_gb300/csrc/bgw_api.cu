@@ -988,8 +988,7 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
 // contiguous (row strides sa, sb; C row stride sc): on tensor cores from digit
 // slices (bgw_dz.cu), in pieces of at most 512 MiB of digits per operand.
 // Short sums stay on the FP64 kernel, which rounds every product on its own
-// scale: the slices' 2^-56 of the rows' largest products is below the rounding
-// of an FP64 sum only once that sum has some tens of terms.
+// scale, and fill neither the 32-wide blocks of the digits nor a tile's time.
 constexpr int kDzMinK = 32;
 cudaError_t row_product(bgw_ctx_s *c, long M, int N, int K, const void *A, long sa, bool conjA, const void *B, long sb,
                         bool conjB, const double *wk, void *C, long sc, double alpha) {

@@ -443,7 +443,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                         long long x = n[q];
                         // the last sum is a fraction of x's unit: bring x up to make room for it
                         const int sh = min(max(__clzll(x < 0 ? ~x : x) - 2, 0), 26);
-                        const long long fr = __float2int_rn(f[q] * 0x1p52f);      // units of 2^-52
+                        // units of 2^-52: up to 2^34 of them where a long sum's terms agree in sign
+                        const long long fr = __float2ll_rn(f[q] * 0x1p52f);
                         x = (x << sh) + (sh >= 16 ? fr << (sh - 16) : fr >> (16 - sh));
                         if (g.alpha == kMinusOne) x = -x;
                         d[h] = fix_out(x, 1086 - 36 - sh + ea + eb);
