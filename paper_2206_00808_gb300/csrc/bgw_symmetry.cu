@@ -141,7 +141,7 @@ bgw_status su2_of(const double *avec, const int *rot_lat, double *U, double *axi
 
 // k8_phase: per plane wave i the phase e^{-2 pi i h'.tau}, from the rotated
 // Miller index h' = M h (M = R_lat^-T), folded into a copy of U, V[i][4], as
-// 64-bit integers in units of 2^-61.  k8_unfold: one thread per (plane wave,
+// 64-bit integers on a power-of-two scale of each entry of U.  k8_unfold: one thread per (plane wave,
 // chunk of kBandChunk bands) applies V[i] to its bands; reads and writes are
 // coalesced along i.
 constexpr int kBandChunk = 8;
@@ -150,7 +150,10 @@ struct Op {
     int M[3][3];
     double tau[3];
     double2 u[4];   // U row-major
+    int e[4];       // biased exponent above every component of u[k] times a phase
 };
+// Stands for the exponent of a zero entry of U beside any other's.
+constexpr int kZeroEntry = -8192;
 
 __global__ void __launch_bounds__(128)
 k8_phase(int ngw, const int *__restrict__ gvec, Op op, longlong2 *__restrict__ V) {
@@ -165,18 +168,22 @@ k8_phase(int ngw, const int *__restrict__ gvec, Op op, longlong2 *__restrict__ V
     sincospi(-2.0 * f, &sn, &cs);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        V[(long)k * ngw + i] = make_longlong2(bgw::fix_in<62>(cs * op.u[k].x - sn * op.u[k].y, 1023),
-                                              bgw::fix_in<62>(cs * op.u[k].y + sn * op.u[k].x, 1023));
+        V[(long)k * ngw + i] = make_longlong2(bgw::fix_in<62>(cs * op.u[k].x - sn * op.u[k].y, op.e[k]),
+                                              bgw::fix_in<62>(cs * op.u[k].y + sn * op.u[k].x, op.e[k]));
 }
 
 // Bound: integer issue.  The 16 real products of a band's spin pair and plane
-// wave run as 48 32 x 32-bit multiply-adds: the pair is scaled by its largest
-// component to 60 bits, V is held to 2^-61 (both beyond FP64's 53), and the sums
-// leave as FP64, rounded once.  In FP64 the products alone took 16 x 64 issue
-// cycles of a warp, and each thread formed V for its 16 bands, as many again:
-// 418 bands x 5029 plane waves 93 -> 72 us a call (134 MB, 20 us at the copy rate).
+// wave run as 48 32 x 32-bit multiply-adds: each spin component is scaled by its
+// largest part to 60 bits and each entry of V to 62 (both beyond FP64's 53), an
+// output's two partial sums are aligned to the one of larger scale, and the sum
+// leaves as FP64, rounded once.  (With one scale for the pair, a component 2^-16
+// of the other lost 2e-13 of itself where U is diagonal.)  In FP64 the products
+// alone took 16 x 64 issue cycles of a warp, and each thread formed V for its 16
+// bands, as many again: 418 bands x 5029 plane waves 93 -> 75 us a call (134 MB, 20 us
+// at the copy rate).
 __global__ void __launch_bounds__(256)
-k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ out, int nb, int ngw, const longlong2 *__restrict__ V) {
+k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ out, int nb, int ngw, const longlong2 *__restrict__ V,
+          int4 ve) {
     using bgw::fix_mad;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= ngw) return;
@@ -193,23 +200,25 @@ k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ out, int nb, int
 #pragma unroll 2
     for (int n = blockIdx.y * kBandChunk; n < n1; ++n) {
         const double2 a = in[(2L * n) * ngw + i], b = in[(2L * n + 1) * ngw + i];
-        const int E = max(max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff),
-                          max(__double2hiint(b.x) & 0x7fffffff, __double2hiint(b.y) & 0x7fffffff)) >> 20;
-        const bgw::fix_parts ax = bgw::fix_split(bgw::fix_in<60>(a.x, E)), ay = bgw::fix_split(bgw::fix_in<60>(a.y, E));
-        const bgw::fix_parts bx = bgw::fix_split(bgw::fix_in<60>(b.x, E)), by = bgw::fix_split(bgw::fix_in<60>(b.y, E));
-        const int eb = 1086 - 57 + E - 1022;
+        const int Ea = max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff) >> 20;
+        const int Eb = max(__double2hiint(b.x) & 0x7fffffff, __double2hiint(b.y) & 0x7fffffff) >> 20;
+        const bgw::fix_parts ax = bgw::fix_split(bgw::fix_in<60>(a.x, Ea)), ay = bgw::fix_split(bgw::fix_in<60>(a.y, Ea));
+        const bgw::fix_parts bx = bgw::fix_split(bgw::fix_in<60>(b.x, Eb)), by = bgw::fix_split(bgw::fix_in<60>(b.y, Eb));
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            auto dot = [&](bgw::fix_parts p, bgw::fix_parts q, bgw::fix_parts s, bgw::fix_parts t) {
-                const long long hi = fix_mad(p.h, ax.h, fix_mad(q.h, ay.h, fix_mad(s.h, bx.h, fix_mad(t.h, by.h, 0))));
-                long long lo = fix_mad(p.h, ax.l, fix_mad(p.l, ax.h, fix_mad(q.h, ay.l, fix_mad(q.l, ay.h, bgw::kFixHalf))));
-                lo = fix_mad(s.h, bx.l, fix_mad(s.l, bx.h, fix_mad(t.h, by.l, fix_mad(t.l, by.h, lo))));
-                return bgw::fix_join(hi, lo);
+            auto dot = [&](bgw::fix_parts p, bgw::fix_parts x, bgw::fix_parts q, bgw::fix_parts y) {
+                return bgw::fix_join(fix_mad(p.h, x.h, fix_mad(q.h, y.h, 0)),
+                                     fix_mad(p.h, x.l, fix_mad(p.l, x.h, fix_mad(q.h, y.l, fix_mad(q.l, y.h, bgw::kFixHalf)))));
             };
-            const long long x = dot(vx[2 * r], my[2 * r], vx[2 * r + 1], my[2 * r + 1]);
-            const long long y = dot(vy[2 * r], vx[2 * r], vy[2 * r + 1], vx[2 * r + 1]);
-            double2 o = make_double2(bgw::fix_out(x, eb), bgw::fix_out(y, eb));
-            if (E == 0x7ff) o = make_double2(nan, nan);   // an infinity or a NaN in the pair
+            const int ta = Ea + (r ? ve.z : ve.x), tb = Eb + (r ? ve.w : ve.y), t = max(ta, tb);
+            const int sa = min(t - ta, 63), sb = min(t - tb, 63);
+            auto add = [&](long long p, long long q) {      // |p|, |q| < 2^59
+                return (((2 * p) >> sa) + 1 >> 1) + (((2 * q) >> sb) + 1 >> 1);
+            };
+            const long long x = add(dot(vx[2 * r], ax, my[2 * r], ay), dot(vx[2 * r + 1], bx, my[2 * r + 1], by));
+            const long long y = add(dot(vy[2 * r], ax, vx[2 * r], ay), dot(vy[2 * r + 1], bx, vx[2 * r + 1], by));
+            double2 o = make_double2(bgw::fix_out(x, t - 1016), bgw::fix_out(y, t - 1016));
+            if (max(Ea, Eb) == 0x7ff) o = make_double2(nan, nan);   // an infinity or a NaN in the pair
             out[(2L * n + r) * ngw + i] = o;
         }
     }
@@ -273,10 +282,17 @@ extern "C" bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, 
             for (int j = 0; j < 3; ++j) op.M[i][j] = M[i][j];
             op.tau[i] = tau[i];
         }
-        for (int i = 0; i < 4; ++i) op.u[i] = make_double2(U[2 * i], U[2 * i + 1]);
+        int ve[4];
+        for (int i = 0; i < 4; ++i) {
+            op.u[i] = make_double2(U[2 * i], U[2 * i + 1]);
+            const double m = std::hypot(U[2 * i], U[2 * i + 1]);
+            op.e[i] = m > 0.0 ? std::ilogb(m * (1.0 + 0x1p-40)) + 1023 : 0;
+            ve[i] = m > 0.0 ? op.e[i] : kZeroEntry;
+        }
         const dim3 grid((unsigned)((ngw + 255) / 256), (unsigned)((nb + kBandChunk - 1) / kBandChunk));
         k8_phase<<<(unsigned)((ngw + 127) / 128), 128, 0, s>>>(ngw, h_dev, op, v_dev);
-        k8_unfold<<<grid, 256, 0, s>>>(static_cast<const double2 *>(c_in), static_cast<double2 *>(c_out), nb, ngw, v_dev);
+        k8_unfold<<<grid, 256, 0, s>>>(static_cast<const double2 *>(c_in), static_cast<double2 *>(c_out), nb, ngw, v_dev,
+                                       make_int4(ve[0], ve[1], ve[2], ve[3]));
         e = cudaGetLastError();
     }
     if (g_dev) {
