@@ -28,6 +28,13 @@
 // pipe ran the update at 0.94 of its rate, 64 ms for 16 x 800^2; now 8.9 ms, of
 // which the update takes 4.6 (bound by its epilogue's integer work), k6_diag 1.7
 // (one SM a matrix) and the digits 0.8.
+//
+// Elimination does not notice a scaling of rows and columns by powers of two, but
+// digits, cut on a scale per row, do: where eps~ = D B D, a large d_k of one factor
+// meets 1/d_k of the other (s_0 2^20 times the others', a metal's head at small q:
+// 7e-14 of the largest entry instead of 1e-15).  So k6_balance takes D out: it
+// finds the power of two nearest 1/sqrt(eps~_GG) for every G, which k6_build
+// applies with S and k6_scale undoes.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -53,18 +60,36 @@ __device__ __forceinline__ Z zfma(Z a, Z b, Z c) {   // a * b + c
     return {fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y))};
 }
 
-// A = I - S chi S in place; chi: [nf][n][n] complex128.
-__global__ void k6_build(double2 *__restrict__ A, const double *__restrict__ s, int n) {
+// Power-of-two scales of eps~ (see above), per matrix: x = 2^e with e nearest
+// -log2(eps~_GG) / 2, and s x and s / x.
+__global__ void k6_balance(const double2 *__restrict__ chi, const double *__restrict__ s, int n,
+                           double *__restrict__ sx, double *__restrict__ sox, int *__restrict__ ex) {
+    const long j = blockIdx.y;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n) return;
+    const double sg = s[g], d = 1.0 - sg * sg * chi[(j * n + g) * (long)n + g].x;
+    int e = 0;
+    if (d > 0.0 && isfinite(d)) e = -((ilogb(d) + 1) >> 1);       // else: a pivot will not be positive
+    ex[j * n + g] = e;
+    sx[j * n + g] = scalbn(sg, e);
+    sox[j * n + g] = scalbn(sg, -e);
+}
+
+// A = X (I - S chi S) X in place; chi: [nf][n][n] complex128.  sx: S X, one
+// vector (stride 0, X = I, ex null) or one per matrix (stride n).
+__global__ void k6_build(double2 *__restrict__ A, const double *__restrict__ sx, int stride,
+                         const int *__restrict__ ex, int n) {
     const long j = blockIdx.z;
     const int r = blockIdx.y;
     double2 *row = A + (j * n + r) * (long)n;
-    const double sr = s[r];
+    sx += j * stride;
+    const double sr = sx[r];
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
         double2 v = row[c];
-        const double f = -sr * s[c];
+        const double f = -sr * sx[c];
         v.x *= f;
         v.y *= f;
-        if (c == r) v.x += 1.0;
+        if (c == r) v.x += ex ? scalbn(1.0, 2 * ex[j * n + r]) : 1.0;
         row[c] = v;
     }
 }
@@ -311,38 +336,67 @@ __global__ void __launch_bounds__(256) k6_writeback_t(double2 *__restrict__ A, i
     }
 }
 
-// W = S eps~^-1 S (mode 1) or eps^-1 = S eps~^-1 S^-1 (mode 2).
-__global__ void k6_scale(double2 *__restrict__ A, const double *__restrict__ s, int n, int inverse_cols) {
+// From the inverse A of X eps~ X: W = S X A X S (mode 1) or eps^-1 = S X A X S^-1
+// (mode 2), with sx = S X and div = S X^-1 (both S, stride 0, where X = I).
+__global__ void k6_scale(double2 *__restrict__ A, const double *__restrict__ sx, const double *__restrict__ div,
+                         int stride, int n, int inverse_cols) {
     const long j = blockIdx.z;
     const int r = blockIdx.y;
     double2 *row = A + (j * n + r) * (long)n;
-    const double sr = s[r];
+    sx += j * stride;
+    div += j * stride;
+    const double sr = sx[r];
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
         double2 v = row[c];
-        const double f = inverse_cols ? sr / s[c] : sr * s[c];
+        const double f = inverse_cols ? sr / div[c] : sr * sx[c];
         v.x *= f;
         v.y *= f;
         row[c] = v;
     }
 }
 
+// v 2^e, exactly; through the exponent field where that can hold it.
+__device__ __forceinline__ double times_pow2(double v, int e) {
+    const int hi = __double2hiint(v), f = (hi >> 20) & 0x7ff;
+    if (f == 0 || f == 0x7ff || f + e < 1 || f + e > 0x7fe) return scalbn(v, e);
+    return __hiloint2double(hi + e * (1 << 20), __double2loint(v));
+}
+
+// eps~^-1 = X A X (mode 0).
+__global__ void k6_unbalance(double2 *__restrict__ A, const int *__restrict__ ex, int n) {
+    const long j = blockIdx.z;
+    const int r = blockIdx.y;
+    double2 *row = A + (j * n + r) * (long)n;
+    const int er = ex[j * n + r];
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
+        const int e = er + ex[j * n + c];
+        if (e == 0) continue;
+        const double2 v = row[c];
+        row[c] = make_double2(times_pow2(v.x, e), times_pow2(v.y, e));
+    }
+}
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Workspace: the panels U and T, s, the error words and, on tensor cores, the
-// digit planes of the panels (2 nf matrices), of P (2 nf) and of P A_KR (nf).
+// digit planes of the panels (2 nf matrices), of P (2 nf) and of P A_KR (nf),
+// and the scales s x, s / x and log2 x of every matrix.
 struct Work {
-    size_t U, T, s, err, panels, p, t, total;
+    size_t U, T, s, err, panels, p, t, sx, sox, ex, total;
     Work(int n, int nf) {
         const size_t panel = sizeof(double2) * (size_t)nf * kB * n;
         U = 0;
         T = panel;
         s = align256(2 * panel);
         err = s + align256(sizeof(double) * (size_t)n);
-        panels = p = t = total = err + 256;
+        panels = p = t = sx = sox = ex = total = err + 256;
         if (n >= kDzMinN) {
             p = panels + bgw::dz_planes_bytes(n, kB, 2 * nf, false);
             t = p + bgw::dz_planes_bytes(kB, kB, 2 * nf, true);
-            total = t + bgw::dz_planes_bytes(n, kB, nf, true);
+            sx = t + bgw::dz_planes_bytes(n, kB, nf, true);
+            sox = sx + align256(sizeof(double) * (size_t)nf * n);
+            ex = sox + align256(sizeof(double) * (size_t)nf * n);
+            total = ex + align256(sizeof(int) * (size_t)nf * n);
         }
     }
 };
@@ -426,13 +480,17 @@ extern "C" bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, 
     e = cudaMemcpyAsync(sd, s, sizeof(double) * ng, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 2 * sizeof(int), st);
     const unsigned rowblocks = (unsigned)((ng + 255) / 256);
+    const bool tensor = ng >= kDzMinN;
+    double *sx = tensor ? reinterpret_cast<double *>(w + o.sx) : sd, *sox = tensor ? reinterpret_cast<double *>(w + o.sox) : sd;
+    int *ex = tensor ? reinterpret_cast<int *>(w + o.ex) : nullptr;
+    const int stride = tensor ? ng : 0;
     if (e == cudaSuccess) {
-        k6_build<<<dim3(rowblocks, ng, nfreq), 256, 0, st>>>(A, sd, ng);
+        if (tensor) k6_balance<<<dim3(rowblocks, nfreq), 256, 0, st>>>(A, sd, ng, sx, sox, ex);
+        k6_build<<<dim3(rowblocks, ng, nfreq), 256, 0, st>>>(A, sx, stride, ex, ng);
         e = cudaGetLastError();
     }
     const unsigned tiles = (unsigned)((ng + kTile - 1) / kTile);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k6_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdateSmem);
-    const bool tensor = ng >= kDzMinN;
     int sms = 148;
     if (tensor && e == cudaSuccess) {
         int dev = 0;
@@ -472,7 +530,10 @@ extern "C" bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, 
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && mode > 0) {
-        k6_scale<<<dim3(rowblocks, ng, nfreq), 256, 0, st>>>(A, sd, ng, mode == 2);
+        k6_scale<<<dim3(rowblocks, ng, nfreq), 256, 0, st>>>(A, sx, sox, stride, ng, mode == 2);
+        e = cudaGetLastError();
+    } else if (e == cudaSuccess && tensor) {
+        k6_unbalance<<<dim3(rowblocks, ng, nfreq), 256, 0, st>>>(A, ex, ng);
         e = cudaGetLastError();
     }
     int flag[2] = {0, 0};
