@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256)
 k5z_rowmax(const double2 *__restrict__ M, int P, int ng, const double *__restrict__ w, int nfreq, int R,
            unsigned *__restrict__ rmax, int *__restrict__ err) {
     __shared__ float sv[kRmF][kRmP];
-    __shared__ float red[8][kRmF][2][kRmG];
+    __shared__ unsigned red[8][kRmF][2][kRmG];
     const int p0 = blockIdx.x * kRmP, g0 = blockIdx.y * kRmG;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = g0 + lane;
@@ -89,15 +89,15 @@ k5z_rowmax(const double2 *__restrict__ M, int P, int ng, const double *__restric
             float s = 0.f;
             if (j < nj && p < P) {
                 const double wv = w[(long)(j0 + j) * P + p];
-                s = wv < 0.0 ? sqrtf((float)(-wv)) : 0.f;
+                s = wv < 0.0 ? sqrtf((float)(-wv)) : wv != wv ? __int_as_float(0x7fffffff) : 0.f;
                 if (wv > 0.0) atomicExch(err, kErrSign);
             }
             sv[j][pp] = s;
         }
         __syncthreads();
-        float mr[kRmF], mi[kRmF];
+        unsigned mr[kRmF], mi[kRmF];          // as bits: order of the values, infinities and NaN above them
 #pragma unroll
-        for (int j = 0; j < kRmF; ++j) mr[j] = mi[j] = 0.f;
+        for (int j = 0; j < kRmF; ++j) mr[j] = mi[j] = 0u;
         for (int pp = warp; pp < kRmP && p0 + pp < P; pp += 8) {
             float ar = 0.f, ai = 0.f;
             if (g < ng) {
@@ -107,8 +107,8 @@ k5z_rowmax(const double2 *__restrict__ M, int P, int ng, const double *__restric
             }
 #pragma unroll
             for (int j = 0; j < kRmF; ++j) {
-                mr[j] = fmaxf(mr[j], sv[j][pp] * ar);
-                mi[j] = fmaxf(mi[j], sv[j][pp] * ai);
+                mr[j] = max(mr[j], __float_as_uint(sv[j][pp] * ar));
+                mi[j] = max(mi[j], __float_as_uint(sv[j][pp] * ai));
             }
         }
 #pragma unroll
@@ -119,10 +119,10 @@ k5z_rowmax(const double2 *__restrict__ M, int P, int ng, const double *__restric
         __syncthreads();
         for (int i = threadIdx.x; i < kRmF * 2 * kRmG; i += 256) {
             const int j = i / (2 * kRmG), c = (i / kRmG) % 2, l = i % kRmG;
-            float m = 0.f;
-            for (int q = 0; q < 8; ++q) m = fmaxf(m, red[q][j][c][l]);
+            unsigned m = 0u;
+            for (int q = 0; q < 8; ++q) m = max(m, red[q][j][c][l]);
             const int gg = g0 + l;
-            if (j < nj && gg < ng && m > 0.f) atomicMax(&rmax[(long)(j0 + j) * R + 2 * gg + c], __float_as_uint(m));
+            if (j < nj && gg < ng && m > 0u) atomicMax(&rmax[(long)(j0 + j) * R + 2 * gg + c], m);
         }
     }
 }
@@ -133,9 +133,11 @@ constexpr int kSpP = 32;   // pairs per block (one K block)
 
 // Exponent of a row from its maximum |Y| (float bits; 0 for an all-zero row):
 // the smallest e with 2^(e-1) >= max (1 + 2^-20), the margin covering the
-// FP32 rounding of the bound.
+// FP32 rounding of the bound.  kFixBad for a row with an infinity or a NaN (or
+// beyond FP32's range): its sums leave as NaN.
 __device__ __forceinline__ int row_exponent(unsigned mb) {
     if (mb == 0u) return 0;
+    if (mb >= 0x7f800000u) return kFixBad;
     const float mm = __fmul_ru(__uint_as_float(mb), 1.0f + 0x1p-20f);
     int k;
     frexpf(mm, &k);   // mm = f 2^k, f in [1/2, 1): mm < 2^k
@@ -311,6 +313,7 @@ __device__ __forceinline__ void fold(const ZParams &zp, int j, int grow, int gco
             const int sh = min(max(__clzll(n < 0 ? ~n : n) - 2, 0), 30);
             const long long x = (n << sh) + __float2ll_rn(a3[c0 + i] * __int_as_float((127 + 16 + sh) << 23));
             d[i] = fix_out(-x, 1086 - 32 - sh + er + ec);
+            if (er == kFixBad || ec == kFixBad) d[i] = __longlong_as_double(0x7ff8000000000000ll);
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) o[i] = __shfl_xor_sync(0xffffffffu, d[i], 1);
