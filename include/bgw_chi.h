@@ -310,8 +310,9 @@ BGW_API bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, con
  * arguments; host-side state is what the captured calls left.  Captured
  * calls must be capture-safe: device-resident inputs (on_device = 1 or
  * pinned host buffers), a device finalize, spheres and q-sets already seen
- * (no new host-to-device metadata copies) and scratch already sized by an
- * identical uncaptured sequence; otherwise the call or bgw_graph_end fails
+ * (no new host-to-device metadata copies; the sphere map of a matrix-element
+ * call is copied at each replay, from memory the context keeps) and scratch
+ * already sized by an identical uncaptured sequence; otherwise the call or bgw_graph_end fails
  * with BGW_E_CUDA and the context can be used uncaptured again.
  */
 BGW_API bgw_status bgw_graph_begin(bgw_ctx ctx);

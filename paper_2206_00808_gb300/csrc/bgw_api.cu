@@ -18,6 +18,7 @@
 #include <cstdio>
 #include <utility>
 #include <cstring>
+#include <list>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -171,6 +172,7 @@ struct bgw_ctx_s {
     DevBuf gmap_tmp;     // dielectric-sphere map of a bgw_mtxel_spinor call
     std::vector<int> gmap_host;      // its contents, while every write of it is known (see put_gmap)
     bool gmap_captured = false;
+    std::list<std::vector<int>> gmap_graph;      // sources of the copies captured in graphs: replays read them
     DevBuf errflag;      // device ints, non-zero after a bounded device wait gave up: [0] of the chi0 and
                          // matrix-element kernels, [1] of a digit product (see dz_err)
     int *dz_err() { return static_cast<int *>(errflag.p) + 1; }
@@ -578,16 +580,24 @@ cudaError_t ensure_mtxel_scratch(bgw_ctx_s *c, const QState &s, int na, int nb2)
 // The call's dielectric-sphere map into gmap_tmp; nothing is copied when it
 // holds these very values already (a third of a small call's host time).  Once
 // a copy has been captured in a graph, its replays write the buffer behind the
-// library's back and every call copies.
+// library's back and every call copies; the graph's copy reads its source at
+// each replay, so it is taken from one that lives as long as the context (one
+// for all captured calls on a sphere).
 cudaError_t put_gmap(bgw_ctx_s *c, const std::vector<int> &gmap) {
-    if (st_capturing(c)) c->gmap_captured = true;
+    const std::vector<int> *src = &gmap;
+    if (st_capturing(c)) {
+        c->gmap_captured = true;
+        auto &kept = c->gmap_graph;
+        auto it = std::find(kept.begin(), kept.end(), gmap);
+        src = it != kept.end() ? &*it : &kept.emplace_back(gmap);
+    }
     if (!c->gmap_captured && c->gmap_tmp.p && c->gmap_host == gmap) return cudaSuccess;
     c->gmap_host.clear();
     cudaError_t e = c->gmap_tmp.ensure(sizeof(int) * gmap.size(), c->st);
     // a pageable source: the copy is stream-ordered and has read the vector
     // when it returns, so the buffer can be refilled by a later call
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->gmap_tmp.p, gmap.data(), sizeof(int) * gmap.size(), cudaMemcpyHostToDevice, c->st);
+        e = cudaMemcpyAsync(c->gmap_tmp.p, src->data(), sizeof(int) * gmap.size(), cudaMemcpyHostToDevice, c->st);
     if (e == cudaSuccess && !c->gmap_captured) c->gmap_host = gmap;
     return e;
 }
