@@ -201,6 +201,14 @@ k_unfix_planes(const int4 *__restrict__ F, const int *__restrict__ scale, int n0
     }
 }
 
+// launch(first band, bands) over pieces of at most kMaxGridYZ bands (the band is
+// a launch's y index).
+template <class F>
+cudaError_t by_bands(int nb, F launch) {
+    for (int b0 = 0; b0 < nb; b0 += kMaxGridYZ) launch(b0, nb - b0 < kMaxGridYZ ? nb - b0 : kMaxGridYZ);
+    return cudaGetLastError();
+}
+
 template <int N>
 cudaError_t yz_fix(const double2 *S, int nb, const Axes &a, int4 *U, int *scale, cudaStream_t st) {
     using Tile = K1Tile<N>;
@@ -209,14 +217,18 @@ cudaError_t yz_fix(const double2 *S, int nb, const Axes &a, int4 *U, int *scale,
         const cudaError_t e = cudaFuncSetAttribute(k1_yz_fix<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k1_yz_fix<N><<<dim3((a.n[0] + Tile::XP - 1) / Tile::XP, nb), Tile::THREADS, smem, st>>>(
-        S, a.n[0], a.w[1], a.w[2], a.s[1], a.s[2], U, scale);
-    return cudaGetLastError();
+    return by_bands(nb, [&](int b0, int n) {
+        const long planes = 2L * b0 * a.n[0];
+        k1_yz_fix<N><<<dim3((a.n[0] + Tile::XP - 1) / Tile::XP, n), Tile::THREADS, smem, st>>>(
+            S + planes * a.w[1] * a.w[2], a.n[0], a.w[1], a.w[2], a.s[1], a.s[2], U + planes * N * N, scale + planes);
+    });
 }
 template <int N>
 cudaError_t fix_planes(void *U, int nb, const Axes &a, int *scale, cudaStream_t st) {
-    k_fix_planes<N><<<dim3(a.n[0], nb), kConvThreads, 0, st>>>(U, scale);
-    return cudaGetLastError();
+    return by_bands(nb, [&](int b0, int n) {
+        const long planes = 2L * b0 * a.n[0];
+        k_fix_planes<N><<<dim3(a.n[0], n), kConvThreads, 0, st>>>(static_cast<int4 *>(U) + planes * N * N, scale + planes);
+    });
 }
 
 #define BGW_FOR_FIX_LEN(n, CALL)          \
@@ -261,9 +273,12 @@ cudaError_t grid_to_fix(void *U, int nb, const Axes &a, int *scale, cudaStream_t
 }
 
 cudaError_t fix_to_grid(const void *F, const int *scale, int nb, const Axes &a, void *U, cudaStream_t st) {
-    k_unfix_planes<<<dim3(a.n[0], nb), kConvThreads, 0, st>>>(static_cast<const int4 *>(F), scale, a.n[0],
-                                                              a.n[1] * a.n[2], static_cast<double2 *>(U));
-    return cudaGetLastError();
+    const int NN = a.n[1] * a.n[2];
+    return by_bands(nb, [&](int b0, int n) {
+        const long planes = 2L * b0 * a.n[0];
+        k_unfix_planes<<<dim3(a.n[0], n), kConvThreads, 0, st>>>(static_cast<const int4 *>(F) + planes * NN, scale + planes,
+                                                                 a.n[0], NN, static_cast<double2 *>(U) + planes * NN);
+    });
 }
 
 }  // namespace bgw

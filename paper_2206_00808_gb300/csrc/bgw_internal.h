@@ -151,6 +151,7 @@ inline size_t mtxel_a_bytes(int nv, int nc, const Axes &a, size_t csize, bool fi
 }
 
 // ---- integer grids (bgw_grid_fix.cu, bgw_zy_fix.cu) -----------------------
+constexpr int kMaxGridYZ = 65535;      // blocks of a launch along y or z
 cudaError_t grid_fix_tables_init();
 cudaError_t zy_fix_tables_init();
 // x pass of wfn_to_grid_f64 (B band components) into S.

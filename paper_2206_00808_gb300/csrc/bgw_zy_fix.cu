@@ -198,8 +198,17 @@ cudaError_t zy_fix_n(const int4 *fv, const int *sv, const int4 *fc, const int *s
     if (in_window(a, 1) && in_window(a, 2)) kern = k2_zy_fix<N, (N > 2 * kWinF + 1)>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile::SMEM);
     if (e != cudaSuccess) return e;
-    const dim3 grid(a.n[0], (nv + Tile::TV - 1) / Tile::TV, (nc + Tile::TC - 1) / Tile::TC);
-    kern<<<grid, Tile::THREADS, Tile::SMEM, st>>>(fv, sv, fc, sc, nv, nc, nc, a.w[1], a.w[2], a.s[1], a.s[2], Bs);
+    // tiles of bands are a launch's y and z index: pieces of at most kMaxGridYZ tiles
+    const long planes = 2L * a.n[0], vol = (long)N * N, out = (long)a.n[0] * a.w[1] * a.w[2];
+    const int vmax = kMaxGridYZ * Tile::TV, cmax = kMaxGridYZ * Tile::TC;
+    for (int v0 = 0; v0 < nv; v0 += vmax)
+        for (int c0 = 0; c0 < nc; c0 += cmax) {
+            const int v = nv - v0 < vmax ? nv - v0 : vmax, c = nc - c0 < cmax ? nc - c0 : cmax;
+            const dim3 grid(a.n[0], (v + Tile::TV - 1) / Tile::TV, (c + Tile::TC - 1) / Tile::TC);
+            kern<<<grid, Tile::THREADS, Tile::SMEM, st>>>(fv + v0 * planes * vol, sv + v0 * planes, fc + c0 * planes * vol,
+                                                          sc + c0 * planes, v, c, nc, a.w[1], a.w[2], a.s[1], a.s[2],
+                                                          Bs + ((long)v0 * nc + c0) * out);
+        }
     return cudaGetLastError();
 }
 
