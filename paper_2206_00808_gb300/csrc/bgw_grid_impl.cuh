@@ -1545,15 +1545,24 @@ static cudaError_t mtxel_batch(const C *uv, const C *uc, int nv, int nc, const A
     if (oct_len(a) && (lanes == 8 || (lanes == 0 && use_coop(a) && use_oct(a)))) {
         // eight lanes per line: fused z+y, then the x pass
         cudaError_t e = cudaSuccess;
-        // pairs per CTA: as many of 4, 2, 1 as leave two CTAs per SM and do not
-        // leave SMs without one
+        // pairs per CTA: 4, 2 or 1, such that two CTAs fit an SM and the launch
+        // still fills the chip.  In FP32 that is most of the SMs (z + y stage, us,
+        // one pair against more: 48^3 1 x 4 pairs 9.6 against 12.4 in 48 CTAs, 3 x 4
+        // 13.1 against 12.4 in 144; 64^3 2 x 4 17.9 against 15.2 in 128).  FP64 with
+        // one pair has three CTAs per SM and its pipe busy: four pairs pay from
+        // twelve waves on (48^3 8 x 13 pairs 699 against 752, 8 x 32 1700 against 1705,
+        // 8 x 40 2137 against 2108; 64^3 8 x 24 2616 against 2651, 8 x 32 3484 against
+        // 3409).
         const size_t ex = sizeof(C) * (size_t)(kOctThreads / 8) * kOctBlock;
         const size_t zp = sizeof(C) * ((((size_t)a.n[1] * (a.w[2] | 1)) + 1) / 2 * 2);
+        constexpr long kMinCtas = BGW_F32 ? 128 : 12 * 2 * 152;
         int tcs = 4;
-        while (tcs > 1 && (ex + tcs * zp > (size_t)110 * 1024 || nc < tcs)) tcs /= 2;
+        while (tcs > 1 && (ex + tcs * zp > (size_t)110 * 1024 || nc < tcs ||
+                           (long)nv * ((nc + tcs - 1) / tcs) * a.n[0] < kMinCtas))
+            tcs = BGW_F32 ? tcs / 2 : 1;
         const size_t zs = ex + tcs * zp;
         BGW_FOR_EACH_OCT_LEN(a.n[2], {
-            auto kern = tcs == 4 ? k2_zy_oct<N, 4> : tcs == 2 ? k2_zy_oct<N, 2> : k2_zy_oct<N, 1>;
+            auto kern = tcs == 4 ? k2_zy_oct<N, 4> : tcs == 2 ? k2_zy_oct<N, BGW_F32 ? 2 : 1> : k2_zy_oct<N, 1>;
             if (zs > 48 * 1024) {
                 e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zs);
                 if (e != cudaSuccess) return e;
