@@ -368,7 +368,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
         const int quarter = warp & 3, group = warp >> 2;
         const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(16 * group);
         long gsub = 0;
-        bool ok = true;
         for (int item = blockIdx.x; item < g.items; item += gridDim.x) {
             const int b = item / per, ti = item % per / g.tb, tj = item % per % g.tb;
             long long n[16];       // sum of orders 0-5 in units of 2^-36,
@@ -379,13 +378,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                 f[i] = 0.f;
             }
             const int nsub = (g.nkb + kSub - 1) / kSub;
-            for (int sub = 0; sub < nsub && ok; ++sub, ++gsub) {
-                bool got = mbar_wait(smem_u32(&set_full), (uint32_t)(gsub & 1));
+            for (int sub = 0; sub < nsub; ++sub, ++gsub) {
+                bool got = !*(volatile int *)&abort_flag && mbar_wait(smem_u32(&set_full), (uint32_t)(gsub & 1));
                 got = __all_sync(0xffffffffu, got && !*(volatile int *)&abort_flag);
                 if (!got) {                     // no further waits: NaN for this tile and the rest
                     if (lane == 0) atomicExch(err, kErrAccum);
                     atomicExch(&abort_flag, 1);
-                    ok = false;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -425,7 +423,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
             const int n0 = (tj * kN + 16 * group) / 2;
             const DzOut &o = g.out;
             if (m < g.M && !(m >= o.skip0 && m < o.skip1)) {
-                const int ea = g.ea[(long)(g.b0a + b) * g.M + m];
+                const int ea = *(volatile int *)&abort_flag ? kFixBad : g.ea[(long)(g.b0a + b) * g.M + m];
                 const int *ebp = g.eb + (long)(g.b0b + b) * g.N;
                 double2 *c = o.c + b * o.sb + m * o.sm + n0 * o.sn;
 #pragma unroll
@@ -450,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dz_gemm(const __grid_constant__
                         d[h] = fix_out(x, 1086 - 36 - sh + ea + eb);
                     }
                     double2 r = make_double2(d[0], d[1]);
-                    if (ea == kFixBad || eb == kFixBad || !ok) r.x = r.y = __longlong_as_double(0x7ff8000000000000ll);
+                    if (ea == kFixBad || eb == kFixBad) r.x = r.y = __longlong_as_double(0x7ff8000000000000ll);
                     if (g.alpha == kComplex)
                         r = make_double2(o.ar * r.x - o.ai * r.y, o.ar * r.y + o.ai * r.x);
                     else if (g.alpha == kReal)
