@@ -20,6 +20,7 @@
 // an improper operation (det = -1) turns the spinor by its proper part -R.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 
@@ -145,6 +146,7 @@ bgw_status su2_of(const double *avec, const int *rot_lat, double *U, double *axi
 // chunk of kBandChunk bands) applies V[i] to its bands; reads and writes are
 // coalesced along i.
 constexpr int kBandChunk = 8;
+constexpr long kMaxBands = 65535L * 16;      // of one call
 
 struct Op {
     int M[3][3];
@@ -196,9 +198,9 @@ k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ out, int nb, int
         my[k] = bgw::fix_split(-v.y);
     }
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    const int n1 = min(nb, (int)(blockIdx.y + 1) * kBandChunk);
+    const int n0 = (blockIdx.z * gridDim.y + blockIdx.y) * kBandChunk, n1 = min(nb, n0 + kBandChunk);
 #pragma unroll 2
-    for (int n = blockIdx.y * kBandChunk; n < n1; ++n) {
+    for (int n = n0; n < n1; ++n) {
         const double2 a = in[(2L * n) * ngw + i], b = in[(2L * n + 1) * ngw + i];
         const int Ea = max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff) >> 20;
         const int Eb = max(__double2hiint(b.x) & 0x7fffffff, __double2hiint(b.y) & 0x7fffffff) >> 20;
@@ -267,7 +269,7 @@ extern "C" bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, 
             gvec_out[3 * g + i] =
                 M[i][0] * gvec_in[3 * g] + M[i][1] * gvec_in[3 * g + 1] + M[i][2] * gvec_in[3 * g + 2];
     if (nb == 0) return BGW_OK;
-    if ((long)nb > 65535L * kBandChunk) return fail(BGW_E_ARG, "unfold_spinor: too many bands for one call");
+    if ((long)nb > kMaxBands) return fail(BGW_E_ARG, "unfold_spinor: too many bands for one call");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     void *g_dev = nullptr;                    // V, then the Miller list
     const size_t gbytes = sizeof(int) * 3 * (size_t)ngw, vbytes = 4 * sizeof(longlong2) * (size_t)ngw;
@@ -289,7 +291,8 @@ extern "C" bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, 
             op.e[i] = m > 0.0 ? std::ilogb(m * (1.0 + 0x1p-40)) + 1023 : 0;
             ve[i] = m > 0.0 ? op.e[i] : kZeroEntry;
         }
-        const dim3 grid((unsigned)((ngw + 255) / 256), (unsigned)((nb + kBandChunk - 1) / kBandChunk));
+        const unsigned chunks = (unsigned)((nb + kBandChunk - 1) / kBandChunk), gy = std::min(chunks, 65535u);
+        const dim3 grid((unsigned)((ngw + 255) / 256), gy, (chunks + gy - 1) / gy);      // y ends at 65535
         k8_phase<<<(unsigned)((ngw + 127) / 128), 128, 0, s>>>(ngw, h_dev, op, v_dev);
         k8_unfold<<<grid, 256, 0, s>>>(static_cast<const double2 *>(c_in), static_cast<double2 *>(c_out), nb, ngw, v_dev,
                                        make_int4(ve[0], ve[1], ve[2], ve[3]));
