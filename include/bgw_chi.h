@@ -291,7 +291,7 @@ BGW_API bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, int
  *   before uploading at k'.  gvec_out is written before the call returns;
  *   c_out when the stream reaches the call.  Uses a stream-ordered device
  *   allocation of 76 ngw bytes (the Miller list and, per plane wave, U with its
- *   phase).  BGW_E_ARG on bad arguments, as for
+ *   phase; the list alone in small calls).  BGW_E_ARG on bad arguments, as for
  *   bgw_symmetry_su2, or aliasing; errors via bgw_last_error(NULL).
  */
 BGW_API bgw_status bgw_symmetry_su2(const double *avec, const int *rot_lat, double *U, double *axis_angle);

@@ -142,11 +142,15 @@ bgw_status su2_of(const double *avec, const int *rot_lat, double *U, double *axi
 
 // k8_phase: per plane wave i the phase e^{-2 pi i h'.tau}, from the rotated
 // Miller index h' = M h (M = R_lat^-T), folded into a copy of U, V[i][4], as
-// 64-bit integers on a power-of-two scale of each entry of U.  k8_unfold: one thread per (plane wave,
-// chunk of kBandChunk bands) applies V[i] to its bands; reads and writes are
-// coalesced along i.
+// 64-bit integers on a power-of-two scale of each entry of U.  k8_unfold: one
+// thread per (plane wave, chunk of kBandChunk bands) applies V[i] (in small calls
+// formed by itself) to its bands; reads and writes are coalesced along i.
 constexpr int kBandChunk = 8;
 constexpr long kMaxBands = 65535L * 16;      // of one call
+// Up to one block per SM, where the launches decide and not the work, each thread
+// forms V itself: a launch and an allocation of 64 bytes per plane wave less
+// (50 bands x 1050 plane waves 63 -> 59 us a call).
+constexpr long kOwnBlocks = 152;
 
 struct Op {
     int M[3][3];
@@ -157,10 +161,7 @@ struct Op {
 // Stands for the exponent of a zero entry of U beside any other's.
 constexpr int kZeroEntry = -8192;
 
-__global__ void __launch_bounds__(128)
-k8_phase(int ngw, const int *__restrict__ gvec, Op op, longlong2 *__restrict__ V) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ngw) return;
+__device__ __forceinline__ void phased(const Op &op, const int *gvec, int i, longlong2 (&v)[4]) {
     const int h0 = gvec[3 * i], h1 = gvec[3 * i + 1], h2 = gvec[3 * i + 2];
     double f = 0;
 #pragma unroll
@@ -170,8 +171,18 @@ k8_phase(int ngw, const int *__restrict__ gvec, Op op, longlong2 *__restrict__ V
     sincospi(-2.0 * f, &sn, &cs);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        V[(long)k * ngw + i] = make_longlong2(bgw::fix_in<62>(cs * op.u[k].x - sn * op.u[k].y, op.e[k]),
-                                              bgw::fix_in<62>(cs * op.u[k].y + sn * op.u[k].x, op.e[k]));
+        v[k] = make_longlong2(bgw::fix_in<62>(cs * op.u[k].x - sn * op.u[k].y, op.e[k]),
+                              bgw::fix_in<62>(cs * op.u[k].y + sn * op.u[k].x, op.e[k]));
+}
+
+__global__ void __launch_bounds__(128)
+k8_phase(int ngw, const int *__restrict__ gvec, Op op, longlong2 *__restrict__ V) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= ngw) return;
+    longlong2 v[4];
+    phased(op, gvec, i, v);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) V[(long)k * ngw + i] = v[k];
 }
 
 // Bound: integer issue.  The 16 real products of a band's spin pair and plane
@@ -183,19 +194,27 @@ k8_phase(int ngw, const int *__restrict__ gvec, Op op, longlong2 *__restrict__ V
 // alone took 16 x 64 issue cycles of a warp, and each thread formed V for its 16
 // bands, as many again: 418 bands x 5029 plane waves 93 -> 75 us a call (134 MB, 20 us
 // at the copy rate).
+// OWN: a thread forms V itself (one launch; see kOwnBlocks).
+template <bool OWN>
 __global__ void __launch_bounds__(256)
 k8_unfold(const double2 *__restrict__ in, double2 *__restrict__ out, int nb, int ngw, const longlong2 *__restrict__ V,
-          int4 ve) {
+          int4 ve, const int *__restrict__ gvec, Op op) {
     using bgw::fix_mad;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= ngw) return;
+    longlong2 v[4];
+    if constexpr (OWN) {
+        phased(op, gvec, i, v);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = V[(long)k * ngw + i];
+    }
     bgw::fix_parts vx[4], vy[4], my[4];                   // re, im, -im
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const longlong2 v = V[(long)k * ngw + i];
-        vx[k] = bgw::fix_split(v.x);
-        vy[k] = bgw::fix_split(v.y);
-        my[k] = bgw::fix_split(-v.y);
+        vx[k] = bgw::fix_split(v[k].x);
+        vy[k] = bgw::fix_split(v[k].y);
+        my[k] = bgw::fix_split(-v[k].y);
     }
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     const int n0 = (blockIdx.z * gridDim.y + blockIdx.y) * kBandChunk, n1 = min(nb, n0 + kBandChunk);
@@ -272,7 +291,10 @@ extern "C" bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, 
     if ((long)nb > kMaxBands) return fail(BGW_E_ARG, "unfold_spinor: too many bands for one call");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     void *g_dev = nullptr;                    // V, then the Miller list
-    const size_t gbytes = sizeof(int) * 3 * (size_t)ngw, vbytes = 4 * sizeof(longlong2) * (size_t)ngw;
+    const unsigned chunks = (unsigned)((nb + kBandChunk - 1) / kBandChunk), gy = std::min(chunks, 65535u);
+    const dim3 grid((unsigned)((ngw + 255) / 256), gy, (chunks + gy - 1) / gy);      // y ends at 65535
+    const bool own = (long)grid.x * chunks <= kOwnBlocks;
+    const size_t gbytes = sizeof(int) * 3 * (size_t)ngw, vbytes = own ? 0 : 4 * sizeof(longlong2) * (size_t)ngw;
     cudaError_t e = cudaMallocAsync(&g_dev, vbytes + gbytes, s);
     longlong2 *v_dev = static_cast<longlong2 *>(g_dev);
     int *h_dev = reinterpret_cast<int *>(static_cast<char *>(g_dev) + vbytes);
@@ -291,11 +313,15 @@ extern "C" bgw_status bgw_unfold_spinor(const double *avec, const int *rot_lat, 
             op.e[i] = m > 0.0 ? std::ilogb(m * (1.0 + 0x1p-40)) + 1023 : 0;
             ve[i] = m > 0.0 ? op.e[i] : kZeroEntry;
         }
-        const unsigned chunks = (unsigned)((nb + kBandChunk - 1) / kBandChunk), gy = std::min(chunks, 65535u);
-        const dim3 grid((unsigned)((ngw + 255) / 256), gy, (chunks + gy - 1) / gy);      // y ends at 65535
-        k8_phase<<<(unsigned)((ngw + 127) / 128), 128, 0, s>>>(ngw, h_dev, op, v_dev);
-        k8_unfold<<<grid, 256, 0, s>>>(static_cast<const double2 *>(c_in), static_cast<double2 *>(c_out), nb, ngw, v_dev,
-                                       make_int4(ve[0], ve[1], ve[2], ve[3]));
+        const double2 *in = static_cast<const double2 *>(c_in);
+        double2 *out = static_cast<double2 *>(c_out);
+        const int4 e4 = make_int4(ve[0], ve[1], ve[2], ve[3]);
+        if (own) {
+            k8_unfold<true><<<grid, 256, 0, s>>>(in, out, nb, ngw, nullptr, e4, h_dev, op);
+        } else {
+            k8_phase<<<(unsigned)((ngw + 127) / 128), 128, 0, s>>>(ngw, h_dev, op, v_dev);
+            k8_unfold<false><<<grid, 256, 0, s>>>(in, out, nb, ngw, v_dev, e4, nullptr, op);
+        }
         e = cudaGetLastError();
     }
     if (g_dev) {
