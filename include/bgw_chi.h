@@ -376,7 +376,9 @@ BGW_API bgw_status bgw_graph_launch(bgw_ctx ctx);
  *                        grids (bgw_mtxel_spinor, bgw_chi0_accumulate,
  *                        bgw_autotune) or to bgw_graph_begin, and the grids of
  *                        all deferred k-points are built together, in one
- *                        launch per 64 k-points where the box and path allow.
+ *                        launch (FP64: two) per 64 k-points where the box and
+ *                        path allow (FP64: integer grids, see bgw_create, as
+ *                        many k-points as 256 MiB of scratch hold).
  *                        A device upload (on_device = 1) then keeps a reference
  *                        to the caller's coefficient buffer until that build:
  *                        keep it alive and unchanged until then; a host upload

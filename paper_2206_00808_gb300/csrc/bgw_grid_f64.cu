@@ -23,8 +23,8 @@ cudaError_t wfn_to_grid_f64(const double *coeff, int ngw, int B, const int *cube
                             const Axes &a, void *S, void *R, void *U, cudaStream_t st, int path) {
     return f64::wfn_to_grid(coeff, ngw, B, cube_map, a, S, R, U, st, path);
 }
-cudaError_t wfn_to_grid_batch_f64(const K1Job *jobs, int n, int B, cudaStream_t st, bool *batched) {
-    return f64::wfn_to_grid_batch(jobs, n, B, st, batched);
+cudaError_t wfn_xpass_batch_f64(const K1Job *jobs, int n, int B, cudaStream_t st) {
+    return f64::wfn_xpass_batch(jobs, n, B, st);
 }
 cudaError_t bounds_take_grid_f64(unsigned *word) {
     unsigned a = 0, b = 0;

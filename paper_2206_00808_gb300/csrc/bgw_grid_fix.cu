@@ -32,15 +32,13 @@ struct K1Tile {
 };
 
 template <int N>
-__global__ void __launch_bounds__(K1Tile<N>::THREADS)
-k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2, int4 *__restrict__ U,
-          int *__restrict__ scale) {
+__device__ __forceinline__ void k1_yz_fix_body(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
+                                               int4 *__restrict__ U, int *__restrict__ scale, long b) {
     constexpr int XP = K1Tile<N>::XP, THREADS = K1Tile<N>::THREADS, RS = K1Tile<N>::RS;
     constexpr int NN = N * N, TOP = fix_top(N), GTOP = fix_grid_top(N);
     extern __shared__ int4 yz_raw[];
     __shared__ int smax[2 * XP], ybits[2 * XP], zbits[2 * XP];      // per (spin component, plane)
     const int x0 = blockIdx.x * XP, xp = min(XP, n0 - x0);
-    const long b = blockIdx.y;
     const int cells = w1 * w2, w2p = w2 | 1;
     // A: [2][XP][w1][w2] inputs, Y: [2][XP][N][w2p] y outputs; C: [2][XP][N][RS]
     // z outputs, over both
@@ -142,6 +140,30 @@ k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2,
     }
 }
 
+template <int N>
+__global__ void __launch_bounds__(K1Tile<N>::THREADS)
+k1_yz_fix(const double2 *__restrict__ S, int n0, int w1, int w2, int s1, int s2, int4 *__restrict__ U,
+          int *__restrict__ scale) {
+    k1_yz_fix_body<N>(S, n0, w1, w2, s1, s2, U, scale, blockIdx.y);
+}
+
+// The same for several k-points, blockIdx.z, from band b0 on.
+struct YzBatch {
+    int n0, b0;
+    struct {
+        const double2 *S;
+        int4 *U;
+        int *scale;
+        int w1, w2, s1, s2;
+    } job[kK1BatchMax];
+};
+template <int N>
+__global__ void __launch_bounds__(K1Tile<N>::THREADS)
+k1_yz_fix_batch(const __grid_constant__ YzBatch jb) {
+    const auto &j = jb.job[blockIdx.z];
+    k1_yz_fix_body<N>(j.S, jb.n0, j.w1, j.w2, j.s1, j.s2, j.U, j.scale, (long)jb.b0 + blockIdx.y);
+}
+
 // FP64 grid -> integer grid in place, one CTA per (x-plane, band).
 template <int N>
 __global__ void __launch_bounds__(kConvThreads)
@@ -224,6 +246,29 @@ cudaError_t yz_fix(const double2 *S, int nb, const Axes &a, int4 *U, int *scale,
     });
 }
 template <int N>
+cudaError_t yz_fix_batch(const K1Job *jobs, int n, int nb, cudaStream_t st) {
+    using Tile = K1Tile<N>;
+    YzBatch jb;
+    jb.n0 = jobs[0].a.n[0];
+    size_t smem = 0;
+    for (int i = 0; i < n; ++i) {
+        const Axes &a = jobs[i].a;
+        jb.job[i] = {static_cast<const double2 *>(jobs[i].S), static_cast<int4 *>(jobs[i].U), jobs[i].scale,
+                     a.w[1], a.w[2], a.s[1], a.s[2]};
+        const size_t s = Tile::smem(a.w[1], a.w[2]);
+        smem = s > smem ? s : smem;
+    }
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k1_yz_fix_batch<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    return by_bands(nb, [&](int b0, int m) {
+        jb.b0 = b0;
+        k1_yz_fix_batch<N><<<dim3((jb.n0 + Tile::XP - 1) / Tile::XP, m, n), Tile::THREADS, smem, st>>>(jb);
+    });
+}
+template <int N>
 cudaError_t fix_planes(void *U, int nb, const Axes &a, int *scale, cudaStream_t st) {
     return by_bands(nb, [&](int b0, int n) {
         const long planes = 2L * b0 * a.n[0];
@@ -263,6 +308,14 @@ cudaError_t wfn_to_fix(const double *coeff, int ngw, int nb, const int *cube_map
     int4 *u = static_cast<int4 *>(U);
 #define BGW_CALL(N) yz_fix<N>(s, nb, a, u, scale, st)
     BGW_FOR_FIX_LEN(a.n[1], BGW_CALL)
+#undef BGW_CALL
+}
+
+cudaError_t wfn_to_fix_batch(const K1Job *jobs, int n, int nb, cudaStream_t st) {
+    const cudaError_t e = wfn_xpass_batch_f64(jobs, n, 2 * nb, st);
+    if (e != cudaSuccess) return e;
+#define BGW_CALL(N) yz_fix_batch<N>(jobs, n, nb, st)
+    BGW_FOR_FIX_LEN(jobs[0].a.n[1], BGW_CALL)
 #undef BGW_CALL
 }
 

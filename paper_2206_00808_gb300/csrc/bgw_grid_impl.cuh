@@ -129,9 +129,9 @@ __device__ __forceinline__ void store_kept(const C (&a)[N], C *o, int stride, in
 // ------------------------------------------------------ sphere -> grid --
 // Pass x: one thread per (band component b, y', z') line of the cube.
 template <int N>
-__global__ void __launch_bounds__(kLineThreads, sizeof(T) == 8 && N <= 24 ? 3 : 0)   // 24^3 FP64: 66 -> 58 us with three CTAs per SM
-k1_xpass(const double2 *__restrict__ coeff, int ngw, long B, const int *__restrict__ cube_map,
-         int w0, int w1, int w2, int s0, C *__restrict__ S) {
+__device__ __forceinline__ void k1_xpass_body(const double2 *__restrict__ coeff, int ngw, long B,
+                                              const int *__restrict__ cube_map, int w0, int w1, int w2, int s0,
+                                              C *__restrict__ S) {
     const long yzs = (long)w1 * w2;
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= B * yzs) return;
@@ -156,6 +156,31 @@ k1_xpass(const double2 *__restrict__ coeff, int ngw, long B, const int *__restri
     C *out = S + b * N * yzs + yz;
 #pragma unroll
     for (int x = 0; x < N; ++x) out[x * yzs] = a[x];
+}
+
+template <int N>
+__global__ void __launch_bounds__(kLineThreads, sizeof(T) == 8 && N <= 24 ? 3 : 0)   // 24^3 FP64: 66 -> 58 us with three CTAs per SM
+k1_xpass(const double2 *__restrict__ coeff, int ngw, long B, const int *__restrict__ cube_map,
+         int w0, int w1, int w2, int s0, C *__restrict__ S) {
+    k1_xpass_body<N>(coeff, ngw, B, cube_map, w0, w1, w2, s0, S);
+}
+
+// The same for several k-points, blockIdx.y.
+struct K1XJob {
+    const double2 *coeff;
+    const int *cube_map;
+    C *S;
+    int ngw, w0, w1, w2, s0;
+};
+struct K1XBatch {
+    long B;
+    K1XJob job[kK1BatchMax];
+};
+template <int N>
+__global__ void __launch_bounds__(kLineThreads, sizeof(T) == 8 && N <= 24 ? 3 : 0)
+k1_xpass_batch(const __grid_constant__ K1XBatch jb) {
+    const K1XJob &j = jb.job[blockIdx.y];
+    k1_xpass_body<N>(j.coeff, j.ngw, jb.B, j.cube_map, j.w0, j.w1, j.w2, j.s0, j.S);
 }
 
 // Pass y: one thread per (b, x, z') line; input rows y' < w1 of S.
@@ -742,7 +767,6 @@ k1_fused(const double2 *__restrict__ coeff, int ngw, const int *__restrict__ inv
 
 // Several k-points in one launch (deferred uploads): CTA x = (job, band
 // component), so the launch has no wave tail per k-point.
-constexpr int kK1BatchMax = 64;
 struct K1BatchJob {
     const double2 *coeff;
     const int *inv;
@@ -1224,6 +1248,23 @@ static cudaError_t wfn_xpass(const double2 *cf, int ngw, long nb, const int *cub
     return cudaGetLastError();
 }
 
+#if !BGW_F32
+static cudaError_t wfn_xpass_batch(const K1Job *jobs, int n, long nb, cudaStream_t st) {
+    K1XBatch jb;
+    jb.B = nb;
+    long lines = 0;
+    for (int i = 0; i < n; ++i) {
+        const K1Job &j = jobs[i];
+        jb.job[i] = K1XJob{reinterpret_cast<const double2 *>(j.coeff), j.cube_map, static_cast<C *>(j.S), j.ngw,
+                           j.a.w[0], j.a.w[1], j.a.w[2], j.a.s[0]};
+        const long l = nb * j.a.w[1] * j.a.w[2];
+        lines = l > lines ? l : lines;
+    }
+    BGW_FOR_EACH_LEN(jobs[0].a.n[0], (k1_xpass_batch<N><<<dim3(blocks_for(lines), n), kLineThreads, 0, st>>>(jb)));
+    return cudaGetLastError();
+}
+#endif
+
 static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *cube_map,
                                const Axes &a, void *S, void *R, void *U, cudaStream_t st, int path) {
     const long nb = B;
@@ -1348,6 +1389,7 @@ static cudaError_t wfn_to_grid(const double *coeff, int ngw, int B, const int *c
     return cudaGetLastError();
 }
 
+#if BGW_F32
 // K1 of several k-points in launches of up to kK1BatchMax: only when every
 // job takes the shared-cube one-kernel transform of the automatic path with
 // the same box (else *batched = false and nothing is launched; the caller
@@ -1392,6 +1434,7 @@ static cudaError_t wfn_to_grid_batch(const K1Job *jobs, int n, int B, cudaStream
     *batched = true;
     return cudaSuccess;
 }
+#endif
 
 #endif
 #if BGW_GRID_PART != 1   // matrix elements

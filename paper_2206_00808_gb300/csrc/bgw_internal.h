@@ -44,11 +44,14 @@ struct K1Job {
     const int *cube_map;      // cube map followed by the inverse map (device)
     Axes a;
     void *U;                  // grid slot [B][n0][n1][n2]
+    // integer grids (wfn_to_fix_batch)
+    void *S = nullptr;        // scratch [B][n0][w1][w2] of this job
+    int *scale = nullptr;
 };
+constexpr int kK1BatchMax = 64;       // k-points of one launch
 // K1 of n k-points in as few launches as possible, when every job takes the
 // shared-cube one-kernel transform with one box length; *batched = false and
 // nothing launched otherwise.
-cudaError_t wfn_to_grid_batch_f64(const K1Job *jobs, int n, int B, cudaStream_t st, bool *batched);
 cudaError_t wfn_to_grid_batch_f32(const K1Job *jobs, int n, int B, cudaStream_t st, bool *batched);
 
 // Pair density, pruned forward FFT and gather for P = nv*nc pairs of one k:
@@ -161,6 +164,9 @@ cudaError_t wfn_xpass_f64(const double *coeff, int ngw, int B, const int *cube_m
 // scale [nb][2][n0].
 cudaError_t wfn_to_fix(const double *coeff, int ngw, int nb, const int *cube_map, const Axes &a, void *S, void *U,
                        int *scale, cudaStream_t st);
+// The same for n <= kK1BatchMax k-points in two launches.
+cudaError_t wfn_xpass_batch_f64(const K1Job *jobs, int n, int B, cudaStream_t st);
+cudaError_t wfn_to_fix_batch(const K1Job *jobs, int n, int nb, cudaStream_t st);
 // FP64 grid to integer grid in place, and an integer grid to an FP64 one.
 cudaError_t grid_to_fix(void *U, int nb, const Axes &a, int *scale, cudaStream_t st);
 cudaError_t fix_to_grid(const void *F, const int *scale, int nb, const Axes &a, void *U, cudaStream_t st);
