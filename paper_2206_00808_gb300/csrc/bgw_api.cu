@@ -1040,7 +1040,10 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
 // contiguous (row strides sa, sb; C row stride sc): on tensor cores from digit
 // slices (bgw_dz.cu), in pieces of at most 512 MiB of digits per operand.
 // Short sums stay on the FP64 kernel, which rounds every product on its own
-// scale, and fill neither the 32-wide blocks of the digits nor a tile's time.
+// scale.  Both forms meet between 16 and 24 terms whatever the number of rows
+// (self-energy call, 18^3 box, 64 pairs, us in FP64 / from digits: 16 G 111 / 114,
+// 32 G 128 / 117, 120 G 237 / 153; BSE block of 4 x 8 pairs 188 / 203, 244 / 216,
+// 562 / 308).
 constexpr int kDzMinK = 32;
 cudaError_t row_product(bgw_ctx_s *c, long M, int N, int K, const void *A, long sa, bool conjA, const void *B, long sb,
                         bool conjB, const double *wk, void *C, long sc, double alpha) {
@@ -1052,15 +1055,19 @@ cudaError_t row_product(bgw_ctx_s *c, long M, int N, int K, const void *A, long 
         return std::min(rows, std::max(128L, (long)(cap / one) / 128 * 128));
     };
     const int mp = (int)piece(M, false), np = (int)piece(N, true);
-    const size_t abytes = bgw::dz_planes_bytes(mp, K, 1, false);
-    cudaError_t e = c->nx_dz.ensure(abytes + bgw::dz_planes_bytes(np, K, 1, true), c->st);
+    const size_t abytes = bgw::dz_planes_bytes(mp, K, 1, false), bbytes = bgw::dz_planes_bytes(np, K, 1, true);
+    cudaError_t e = c->nx_dz.ensure(abytes + bbytes + bgw::dz_balance_bytes(K), c->st);
     char *ws = static_cast<char *>(c->nx_dz.p);
-    const double2 *a = static_cast<const double2 *>(A), *b = static_cast<const double2 *>(B);
+    bgw::DzOperand a = {static_cast<const double2 *>(A), 0, sa, 1, conjA, wk};
+    bgw::DzOperand b = {static_cast<const double2 *>(B), 0, sb, 1, conjB, nullptr};
+    if (e == cudaSuccess) e = bgw::dz_balance(a, M, b, N, K, ws + abytes + bbytes, c->st);
     for (int n0 = 0; n0 < N && e == cudaSuccess; n0 += np)
         for (long m0 = 0; m0 < M && e == cudaSuccess; m0 += mp) {
             const int m = (int)std::min<long>(mp, M - m0), n = std::min(np, N - n0);
             const bgw::DzPlanes pl[2] = {bgw::dz_planes(ws, m, K, 1, false), bgw::dz_planes(ws + abytes, n, K, 1, true)};
-            const bgw::DzOperand op[2] = {{a + m0 * sa, 0, sa, 1, conjA, wk}, {b + (long)n0 * sb, 0, sb, 1, conjB, nullptr}};
+            bgw::DzOperand op[2] = {a, b};
+            op[0].p += m0 * sa;
+            op[1].p += (long)n0 * sb;
             e = bgw::dz_split(op, pl, 2, K, c->st);
             const bgw::DzOut out = {static_cast<double2 *>(C) + m0 * sc + n0, 0, sc, 1, 0, 0, alpha, 0.0, false};
             if (e == cudaSuccess)

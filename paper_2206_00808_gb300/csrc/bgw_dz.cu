@@ -10,6 +10,11 @@
 // largest entries meet small ones (W near G = 0, orthogonal states there) keep
 // nine bits in hand.  (Seven digits and 28 products had the error of FP64 sums
 // or up to a third more on such rows.)
+// Where one operand's entries rise along k as the other's fall (v(G) in W against
+// matrix elements that vanish with G -> 0), scales per row cut off what the other
+// makes up for: dz_balance finds each column's largest entry relative to its rows
+// and the split moves half the difference of the two operands, a power of two per
+// k, from one to the other.
 // Products of one order t + u are integers in units of 2^(-8(t+u)); over 160 k
 // the sums of orders 0 to 5 (1 to 6 products of at most 2^14) stay below 2^24
 // units, so an FP32 accumulator in TMEM holds them exactly; they are moved to
@@ -74,8 +79,8 @@ struct SplitArgs {
 };
 
 // Element (row, k) of an operand, weight and conjugation applied.
-__device__ __forceinline__ double2 dz_load(const DzOperand &op, const double2 *base, int row, int k) {
-    double2 v = base[row * op.sr + k * op.sk];
+__device__ __forceinline__ double2 dz_load(const DzOperand &op, const double2 *base, long row, int k) {
+    double2 v = __ldg(base + row * op.sr + k * op.sk);
     if (op.w) {
         const double w = op.w[k];
         v.x *= w;
@@ -106,10 +111,67 @@ __device__ __forceinline__ void dz_store(__nv_bfloat16 *x, long plane, const lon
     }
 }
 
-// 32 rows of one operand per block, every k.
+// Exponent of a value's larger component for the comparisons below.
+constexpr int kExpZero = -4096, kExpBad = 1 << 20;      // zero or subnormal; not finite
+__device__ __forceinline__ int dz_exponent(double2 v) {
+    const int e = max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) >> 20;
+    return e == 0 ? kExpZero : e == 0x7ff ? kExpBad : e;
+}
+// Power of two that column k of this operand is multiplied by.
+__device__ __forceinline__ int dz_shift(const DzOperand &op, int k) {
+    if (!op.cols) return 0;
+    const int c = op.cols[k], o = op.other[k];
+    if (c <= kExpZero || o <= kExpZero) return 0;
+    return op.second ? -((c - o) >> 1) : (o - c) >> 1;
+}
+
+// Column exponents of both operands of a product, each entry's taken relative to
+// its row's largest: a block has kBalRows rows, a warp each, and keeps their
+// entries' exponents in shared memory [row][K] for the columns.  Bound: one
+// latency of the operands' read and the launch.
+constexpr int kBalRows = 8;
+struct BalanceArgs {
+    DzOperand op[2];
+    long rows[2];
+    int *col[2];
+    int K;
+};
+__global__ void __launch_bounds__(32 * kBalRows) k_dz_balance(const __grid_constant__ BalanceArgs a) {
+    extern __shared__ short ex[];
+    __shared__ int er[kBalRows];
+    const long groups0 = (a.rows[0] + kBalRows - 1) / kBalRows;
+    const int w = blockIdx.x >= groups0, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const DzOperand op = a.op[w];
+    const long row = (w ? blockIdx.x - groups0 : blockIdx.x) * kBalRows + warp;
+    const bool there = row < a.rows[w];
+    const double2 *base = op.p + (there ? row : 0) * op.sr;
+    int m = kExpZero;
+#pragma unroll 4
+    for (int k = lane; k < a.K; k += 32) {
+        const int e = there ? dz_exponent(dz_load(op, base, 0, k)) : kExpZero;
+        m = max(m, e);
+        ex[warp * a.K + k] = (short)min(e, 0x7fff);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) er[warp] = m;
+    __syncthreads();
+    for (int k = threadIdx.x; k < a.K; k += 32 * kBalRows) {
+        int c = kExpZero;
+#pragma unroll
+        for (int i = 0; i < kBalRows; ++i) {
+            const int e = ex[i * a.K + k];
+            if (er[i] != kExpBad && e != kExpZero) c = max(c, e - er[i]);      // a row that is not finite has no say
+        }
+        if (c > *(volatile int *)&a.col[w][k]) atomicMax(&a.col[w][k], c);
+    }
+}
+
+// 32 rows of one operand per block, a part of their k' blocks each along y (every
+// block finds its rows' largest entries itself).
 __global__ void __launch_bounds__(kSpThreads) k_dz_split(const __grid_constant__ SplitArgs a) {
     __shared__ double2 sm[kSpRows][kKB / 2 + 1];
     __shared__ int smax[kSpRows];
+    extern __shared__ int shift[];                    // of every k
     int w = 0;
     while (w + 1 < a.n && blockIdx.x >= a.o[w + 1].first) ++w;
     const SplitOp &o = a.o[w];
@@ -119,39 +181,55 @@ __global__ void __launch_bounds__(kSpThreads) k_dz_split(const __grid_constant__
     const double2 *base = o.op.p + b * o.op.sb;
     const bool along_rows = o.op.sr == 1;             // consecutive lanes take consecutive rows
     const int t = threadIdx.x;
-    if (t < kSpRows) smax[t] = 0;
+    if (t < kSpRows) smax[t] = kExpZero;
+    for (int k = t; k < a.K; k += kSpThreads) shift[k] = dz_shift(o.op, k);
     __syncthreads();
     // the rows' largest components
     if (along_rows) {
         const int row = r0 + t % kSpRows;
-        int m = 0;
+        int m = kExpZero;
         if (row < o.rows)
-            for (int k = t / kSpRows; k < a.K; k += kSpThreads / kSpRows) {
-                const double2 v = dz_load(o.op, base, row, k);
-                m = max(m, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
-            }
+            for (int k = t / kSpRows; k < a.K; k += kSpThreads / kSpRows)
+                m = max(m, dz_exponent(dz_load(o.op, base, row, k)) + shift[k]);
         atomicMax(&smax[t % kSpRows], m);
     } else {
-        for (int rr = t / 32; rr < kSpRows; rr += kSpThreads / 32) {
-            int m = 0;
-            if (r0 + rr < o.rows)
-                for (int k = t % 32; k < a.K; k += 32) {
-                    const double2 v = dz_load(o.op, base, r0 + rr, k);
-                    m = max(m, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
-                }
-            m = __reduce_max_sync(0xffffffffu, m);
-            if (t % 32 == 0) smax[rr] = m;
+        // a warp's rows together, for as many loads in flight
+        constexpr int kWarps = kSpThreads / 32, kPer = kSpRows / kWarps;
+        int m[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) m[i] = kExpZero;
+#pragma unroll 2
+        for (int k = t % 32; k < a.K; k += 32)
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int row = min(r0 + t / 32 + kWarps * i, o.rows - 1);
+                m[i] = max(m[i], dz_exponent(dz_load(o.op, base, row, k)) + shift[k]);
+            }
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+            if (t % 32 == 0) smax[t / 32 + kWarps * i] = m[i];
         }
     }
     __syncthreads();
-    if (t < kSpRows && r0 + t < o.rows) {
-        const int E = smax[t] >> 20;
-        o.scale[(long)(o.batch0 + b) * o.rows + r0 + t] = E == 0x7ff ? kFixBad : E - 1022 - kTopD + 8 * (kSl - 1);
+    if (blockIdx.y == 0 && t < kSpRows && r0 + t < o.rows) {
+        const int E = smax[t];
+        o.scale[(long)(o.batch0 + b) * o.rows + r0 + t] = E >= kExpBad / 2 ? kFixBad : E - 1022 - kTopD + 8 * (kSl - 1);
     }
     const int rr = t / 8, seg = t % 8;                // this thread's row and pair of complex values
-    const int E = smax[rr] >> 20;
+    const int E = smax[rr];
     const long plane = o.tiles * kM * (long)a.kblocks * kKB;
-    for (int kb = 0; kb < a.kblocks; ++kb) {
+    auto fetch = [&](int kb, double2 (&v)[2]) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int kk = kb * (kKB / 2) + 2 * seg + i;
+            v[i] = r0 + rr < o.rows && kk < a.K ? dz_load(o.op, base, r0 + rr, kk) : make_double2(0.0, 0.0);
+        }
+    };
+    const int kb0 = a.kblocks * (int)blockIdx.y / (int)gridDim.y, kb1 = a.kblocks * (int)(blockIdx.y + 1) / (int)gridDim.y;
+    double2 ahead[2];
+    if (!along_rows) fetch(kb0, ahead);
+    for (int kb = kb0; kb < kb1; ++kb) {
         double2 v[2];
         if (along_rows) {
             __syncthreads();
@@ -164,17 +242,17 @@ __global__ void __launch_bounds__(kSpThreads) k_dz_split(const __grid_constant__
             v[0] = sm[rr][2 * seg];
             v[1] = sm[rr][2 * seg + 1];
         } else {
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int kk = kb * (kKB / 2) + 2 * seg + i;
-                v[i] = r0 + rr < o.rows && kk < a.K ? dz_load(o.op, base, r0 + rr, kk) : make_double2(0.0, 0.0);
-            }
+            v[0] = ahead[0];
+            v[1] = ahead[1];
+            if (kb + 1 < kb1) fetch(kb + 1, ahead);
         }
         long long n[4];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            n[2 * i] = fix_in<kTopD>(v[i].x, E);
-            n[2 * i + 1] = fix_in<kTopD>(v[i].y, E);
+            const int kk = kb * (kKB / 2) + 2 * seg + i;
+            const int s = kk < a.K ? E - shift[kk] : E;
+            n[2 * i] = fix_in<kTopD>(v[i].x, s);
+            n[2 * i + 1] = fix_in<kTopD>(v[i].y, s);
         }
         if (o.b) {
             const long row = (long)(o.batch0 + b) * o.rows_pad + 2 * (r0 + rr);
@@ -507,6 +585,33 @@ size_t dz_planes_bytes(int rows, int K, int batch, bool b) {
     return plane_bytes(p) + align256(sizeof(int) * (size_t)batch * rows);
 }
 
+size_t dz_balance_bytes(int K) { return align256(sizeof(int) * 2 * (size_t)K); }
+
+cudaError_t dz_balance(DzOperand &A, long rowsA, DzOperand &B, long rowsB, int K, void *ws, cudaStream_t st) {
+    BalanceArgs a;
+    a.op[0] = A;
+    a.op[1] = B;
+    a.rows[0] = rowsA;
+    a.rows[1] = rowsB;
+    a.col[0] = static_cast<int *>(ws);
+    a.col[1] = a.col[0] + K;
+    a.K = K;
+    const size_t smem = sizeof(short) * kBalRows * (size_t)K;
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024)
+        e = cudaFuncSetAttribute(k_dz_balance, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // every byte 0x80: far below kExpZero
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0x80, sizeof(int) * 2 * (size_t)K, st);
+    if (e != cudaSuccess) return e;
+    const long blocks = (rowsA + kBalRows - 1) / kBalRows + (rowsB + kBalRows - 1) / kBalRows;
+    k_dz_balance<<<(unsigned)blocks, 32 * kBalRows, smem, st>>>(a);
+    A.cols = B.other = a.col[0];
+    B.cols = A.other = a.col[1];
+    A.second = false;
+    B.second = true;
+    return cudaGetLastError();
+}
+
 cudaError_t dz_split(const DzOperand *op, const DzPlanes *pl, int n, int K, cudaStream_t st) {
     if (n < 1 || n > kMaxOps) return cudaErrorInvalidValue;
     SplitArgs a;
@@ -520,7 +625,11 @@ cudaError_t dz_split(const DzOperand *op, const DzPlanes *pl, int n, int K, cuda
                          p.first, tile_rows(p) / kM, blocks};
         blocks += (unsigned)(p.used * (p.rows_pad / (p.b ? 2 * kSpRows : kSpRows)));
     }
-    k_dz_split<<<blocks, kSpThreads, 0, st>>>(a);
+    // few rows: the k' blocks of a row, at least two at a time, go to as many thread
+    // blocks as give every SM two (7 x 21 pairs of 350 G: 44 -> 24 us a launch)
+    const int parts = (int)(2 * 152 / blocks), most = a.kblocks / 2;
+    const int y = parts < 1 || most < 1 ? 1 : parts < most ? parts : most;
+    k_dz_split<<<dim3(blocks, y), kSpThreads, sizeof(int) * (size_t)K, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -8,12 +8,15 @@
 namespace bgw {
 
 // Operand (b, row, k) at p[b * sb + row * sr + k * sk], complex128; w: a real
-// weight per k (may be null).
+// weight per k (may be null); cols, other: column exponents of this operand and
+// of the other of its product, from dz_balance (null: none).
 struct DzOperand {
     const double2 *p;
     long sb, sr, sk;
     bool conj;
     const double *w;
+    const int *cols = nullptr, *other = nullptr;
+    bool second = false;     // the B operand: takes the opposite shift
 };
 
 // Digit planes of one operand for `batch` matrices of `rows` rows: an A
@@ -41,6 +44,11 @@ constexpr int kDzMaxK = 5000;
 size_t dz_planes_bytes(int rows, int K, int batch, bool b);
 // Describe planes of `rows` x K in ws (dz_planes_bytes long).
 DzPlanes dz_planes(void *ws, int rows, int K, int batch, bool b);
+// Column exponents of the operands of one product (batch 1, k contiguous): the
+// largest exponent of each column over the rows, each taken relative to its row's
+// largest entry.  ws: dz_balance_bytes long.  Sets cols, other and second of both.
+size_t dz_balance_bytes(int K);
+cudaError_t dz_balance(DzOperand &A, long rowsA, DzOperand &B, long rowsB, int K, void *ws, cudaStream_t st);
 // Cut n operands into their digits, one launch (all of the same K).
 cudaError_t dz_split(const DzOperand *op, const DzPlanes *pl, int n, int K, cudaStream_t st);
 // err: device int, set non-zero when a bounded device wait gave up (the outputs
