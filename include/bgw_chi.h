@@ -440,8 +440,10 @@ BGW_API bgw_status bgw_graph_launch(bgw_ctx ctx);
  *                        resources and records an error that a host finalize
  *                        reports as BGW_E_TIMEOUT; 2, the same for the streamed
  *                        z + y kernel of FP32 32^3 boxes (whose planes arrive by
- *                        TMA): its first CTA skips one plane copy.  No fault,
- *                        trap or hang.
+ *                        TMA): its first CTA skips one plane copy.  For
+ *                        bgw_epsinv, which has no context, the environment
+ *                        variable BGW_FAULT=drop@epsinv does it (from 96 rows
+ *                        on).  No fault, trap or hang.
  */
 enum { BGW_OPT_KCHUNK = 1, BGW_OPT_PAIR_TILE_V = 2, BGW_OPT_PAIR_TILE_C = 3, BGW_OPT_GRID_SLOTS = 4,
        BGW_OPT_TEST_DROP_LOAD = 5, BGW_OPT_TEST_FAIL_ALLOC = 6, BGW_OPT_K1_PATH = 7,

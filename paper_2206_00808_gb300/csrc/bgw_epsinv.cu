@@ -38,6 +38,8 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdlib>
+#include <cstring>
 #include <string>
 
 #include "../../include/bgw_chi.h"
@@ -48,8 +50,10 @@ namespace {
 constexpr int kB = 32;           // Gauss-Jordan block
 constexpr int kTile = 32;        // update tile (rows and columns): many CTAs per panel step
 constexpr int kErrPivot = 1;
-// Rows from which the products run on tensor cores: below, a step's products
-// fill neither form of the kernels and the extra launches decide.
+// Rows from which the products run on tensor cores.  One matrix of 96 rows: 566 us
+// a call in FP64, 454 from digits; 160 917 / 725, 16 matrices of 224 rows 2637 /
+// 1139.  (Digits are also faster below, 64 rows 396 / 323 us and 48 rows 314 / 275,
+// where a call is launches and k6_diag; small matrices keep their workspace.)
 constexpr int kDzMinN = 96;
 
 struct Z {
@@ -497,6 +501,8 @@ extern "C" bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, 
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
+    const char *fault = std::getenv("BGW_FAULT");      // test hook: the first product loses an operand load
+    const bool drop = fault && !std::strcmp(fault, "drop@epsinv");
     for (int k0 = 0; k0 < ng && e == cudaSuccess; k0 += kB) {
         const int kb = ng - k0 < kB ? ng - k0 : kB;
         k6_diag<<<nfreq, 256, 0, st>>>(A, ng, k0, kb, err);
@@ -514,7 +520,8 @@ extern "C" bgw_status bgw_epsinv(int ng, int nfreq, const double *s, void *chi, 
             bgw::DzPlanes both = pa, bothp = bp;
             both.used = bothp.used = 2 * nfreq;
             if (e == cudaSuccess)
-                e = bgw::dz_gemm(both, bothp, bgw::DzOut{U, (long)ng * kB, kB, 1, 0, 0, 1.0, 0.0, false}, sms, st, err + 1);
+                e = bgw::dz_gemm(both, bothp, bgw::DzOut{U, (long)ng * kB, kB, 1, 0, 0, 1.0, 0.0, false}, sms, st, err + 1,
+                                 drop && k0 == 0);
             const bgw::DzPlanes bt = bgw::dz_planes(w + o.t, ng, kB, nfreq, true);
             const bgw::DzOperand ot = {T, (long)ng * kB, kB, 1, false, nullptr};
             if (e == cudaSuccess) e = bgw::dz_split(&ot, &bt, 1, kb, st);
