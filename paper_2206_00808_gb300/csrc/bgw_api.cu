@@ -1038,7 +1038,8 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
 
 // C[m][n] = alpha sum_k opA[m][k] wk[k] opB[n][k] with rows of both operands
 // contiguous (row strides sa, sb; C row stride sc): on tensor cores from digit
-// slices (bgw_dz.cu), in pieces of at most 512 MiB of digits per operand.
+// slices (bgw_dz.cu), in pieces of at most 512 MiB of digits per operand.  Clears
+// the products' error word before it starts.
 // Short sums stay on the FP64 kernel, which rounds every product on its own
 // scale.  Both forms meet between 16 and 24 terms whatever the number of rows
 // (self-energy call, 18^3 box, 64 pairs, us in FP64 / from digits: 16 G 111 / 114,
@@ -1047,8 +1048,11 @@ bgw_status mtxel_into(bgw_ctx_s *c, const char *who, QState &s, int ik, int a0, 
 constexpr int kDzMinK = 32;
 cudaError_t row_product(bgw_ctx_s *c, long M, int N, int K, const void *A, long sa, bool conjA, const void *B, long sb,
                         bool conjB, const double *wk, void *C, long sc, double alpha) {
-    if (K < kDzMinK || K > bgw::kDzMaxK)
-        return bgw::zgemm_f64((int)M, N, K, A, sa, 1, conjA, B, 1, sb, conjB, wk, C, sc, 1, alpha, 0.0, false, c->st);
+    if (K < kDzMinK || K > bgw::kDzMaxK) {
+        const cudaError_t e = cudaMemsetAsync(c->dz_err(), 0, sizeof(int), c->st);
+        return e != cudaSuccess ? e : bgw::zgemm_f64((int)M, N, K, A, sa, 1, conjA, B, 1, sb, conjB, wk, C, sc, 1, alpha,
+                                                     0.0, false, c->st);
+    }
     const size_t cap = (size_t)512 << 20;
     auto piece = [&](long rows, bool b) {
         const size_t one = bgw::dz_planes_bytes(128, K, 1, b) / 128 + 1;
@@ -1060,7 +1064,7 @@ cudaError_t row_product(bgw_ctx_s *c, long M, int N, int K, const void *A, long 
     char *ws = static_cast<char *>(c->nx_dz.p);
     bgw::DzOperand a = {static_cast<const double2 *>(A), 0, sa, 1, conjA, wk};
     bgw::DzOperand b = {static_cast<const double2 *>(B), 0, sb, 1, conjB, nullptr};
-    if (e == cudaSuccess) e = bgw::dz_balance(a, M, b, N, K, ws + abytes + bbytes, c->st);
+    if (e == cudaSuccess) e = bgw::dz_balance(a, M, b, N, K, ws + abytes + bbytes, c->dz_err(), c->st);
     for (int n0 = 0; n0 < N && e == cudaSuccess; n0 += np)
         for (long m0 = 0; m0 < M && e == cudaSuccess; m0 += mp) {
             const int m = (int)std::min<long>(mp, M - m0), n = std::min(np, N - n0);
@@ -2043,7 +2047,6 @@ bgw_status bgw_sigma_cohsex(bgw_ctx c, const bgw_q *q, int ik, int n0, int nn, c
     if (st != BGW_OK) return st;
     double *sw = static_cast<double *>(c->nx_s.p), *tv = sw + P, *out = tv + P;
     e = cudaMemcpyAsync(c->nx_v.p, vq, sizeof(double) * s.ng, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->dz_err(), 0, sizeof(int), c->st);
     // Y[p][G] = sum_G' W[G][G'] M[p][G']
     if (e == cudaSuccess)
         e = row_product(c, P, s.ng, s.ng, c->nx_m1.p, s.ng, false, W_dev, s.ng, false, nullptr, c->nx_y.p, s.ng, 1.0);
@@ -2105,7 +2108,6 @@ bgw_status bgw_bse_kernel(bgw_ctx c, int ik, int jk, const bgw_q *q0, const doub
         if (st == BGW_OK) st = mtxel_into(c, "bse_kernel", s, jk, va, nv, ca, nc, c->nx_m2.p, clean);
         if (st != BGW_OK) return st;
         e = cudaMemcpyAsync(c->nx_v.p, v0_coul, sizeof(double) * s.ng, cudaMemcpyHostToDevice, c->st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->dz_err(), 0, sizeof(int), c->st);
         // KX[I][J] = (1/N_k) sum_G v(G) M_I(k_i, G) conj(M_J(k_j, G))
         if (e == cudaSuccess)
             e = row_product(c, P, (int)P, s.ng, c->nx_m1.p, s.ng, false, c->nx_m2.p, s.ng, true,

@@ -134,6 +134,7 @@ struct BalanceArgs {
     DzOperand op[2];
     long rows[2];
     int *col[2];
+    int *err;
     int K;
 };
 __global__ void __launch_bounds__(32 * kBalRows) k_dz_balance(const __grid_constant__ BalanceArgs a) {
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(32 * kBalRows) k_dz_balance(const __grid_const
     __shared__ int er[kBalRows];
     const long groups0 = (a.rows[0] + kBalRows - 1) / kBalRows;
     const int w = blockIdx.x >= groups0, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.err = 0;
     const DzOperand op = a.op[w];
     const long row = (w ? blockIdx.x - groups0 : blockIdx.x) * kBalRows + warp;
     const bool there = row < a.rows[w];
@@ -587,7 +589,7 @@ size_t dz_planes_bytes(int rows, int K, int batch, bool b) {
 
 size_t dz_balance_bytes(int K) { return align256(sizeof(int) * 2 * (size_t)K); }
 
-cudaError_t dz_balance(DzOperand &A, long rowsA, DzOperand &B, long rowsB, int K, void *ws, cudaStream_t st) {
+cudaError_t dz_balance(DzOperand &A, long rowsA, DzOperand &B, long rowsB, int K, void *ws, int *err, cudaStream_t st) {
     BalanceArgs a;
     a.op[0] = A;
     a.op[1] = B;
@@ -595,12 +597,14 @@ cudaError_t dz_balance(DzOperand &A, long rowsA, DzOperand &B, long rowsB, int K
     a.rows[1] = rowsB;
     a.col[0] = static_cast<int *>(ws);
     a.col[1] = a.col[0] + K;
+    a.err = err;
     a.K = K;
     const size_t smem = sizeof(short) * kBalRows * (size_t)K;
     cudaError_t e = cudaSuccess;
     if (smem > 48 * 1024)
         e = cudaFuncSetAttribute(k_dz_balance, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    // every byte 0x80: far below kExpZero
+    // every byte 0x80: far below kExpZero.  (Cleared by the product before it instead,
+    // at the start of its k_dz_gemm, the products took 7 us longer each.)
     if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0x80, sizeof(int) * 2 * (size_t)K, st);
     if (e != cudaSuccess) return e;
     const long blocks = (rowsA + kBalRows - 1) / kBalRows + (rowsB + kBalRows - 1) / kBalRows;

@@ -46,9 +46,10 @@ size_t dz_planes_bytes(int rows, int K, int batch, bool b);
 DzPlanes dz_planes(void *ws, int rows, int K, int batch, bool b);
 // Column exponents of the operands of one product (batch 1, k contiguous): the
 // largest exponent of each column over the rows, each taken relative to its row's
-// largest entry.  ws: dz_balance_bytes long.  Sets cols, other and second of both.
+// largest entry.  ws: dz_balance_bytes long.  Sets cols, other and second of both,
+// and *err = 0.
 size_t dz_balance_bytes(int K);
-cudaError_t dz_balance(DzOperand &A, long rowsA, DzOperand &B, long rowsB, int K, void *ws, cudaStream_t st);
+cudaError_t dz_balance(DzOperand &A, long rowsA, DzOperand &B, long rowsB, int K, void *ws, int *err, cudaStream_t st);
 // Cut n operands into their digits, one launch (all of the same K).
 cudaError_t dz_split(const DzOperand *op, const DzPlanes *pl, int n, int K, cudaStream_t st);
 // err: device int, set non-zero when a bounded device wait gave up (the outputs
