@@ -25,8 +25,8 @@
 // cores from BF16 digits (bgw_dz.cu, more exact than FP64 sums): the digits of
 // A_RK, of A_KR and of P both ways, one product for both panels (as 2 nf
 // matrices), the digits of P A_KR, and one product for the update.  The FP64
-// pipe ran the update at 0.94 of its rate, 64 ms for 16 x 800^2; now 8.9 ms, of
-// which the update takes 4.6 (bound by its epilogue's integer work), k6_diag 1.7
+// pipe ran the update at 0.94 of its rate, 64 ms for 16 x 800^2; now 9.1 ms, of
+// which the update takes 4.6 (bound by its epilogue's integer work), k6_diag 2.0
 // (one SM a matrix) and the digits 0.8.
 //
 // Elimination does not notice a scaling of rows and columns by powers of two, but
@@ -52,8 +52,9 @@ constexpr int kTile = 32;        // update tile (rows and columns): many CTAs pe
 constexpr int kErrPivot = 1;
 // Rows from which the products run on tensor cores.  One matrix of 96 rows: 566 us
 // a call in FP64, 454 from digits; 160 917 / 725, 16 matrices of 224 rows 2637 /
-// 1139.  (Digits are also faster below, 64 rows 396 / 323 us and 48 rows 314 / 275,
-// where a call is launches and k6_diag; small matrices keep their workspace.)
+// 1139 (with a k6_diag 8 us a block faster).  (Digits are also faster below, 64
+// rows 396 / 323 us and 48 rows 314 / 275, where a call is launches and k6_diag;
+// small matrices keep their workspace.)
 constexpr int kDzMinN = 96;
 
 struct Z {
@@ -103,7 +104,11 @@ __global__ void k6_build(double2 *__restrict__ A, const double *__restrict__ sx,
 // per thread.  Bound: the FP64 pipe of one SM, 4 kb^2 operations a pivot; the
 // reciprocal of the next pivot is formed by the one thread that updates it
 // while the others still update (every thread forming its own took 175 us a
-// call of 16 blocks).
+// call of 16 blocks).  The products of an update are summed before they meet the
+// entry, which is then rounded once: two fused multiply-adds onto it round it
+// twice, for half as much error again in the inverse (95 rows 5.1e-16 against
+// 3.4e-16).  The scaled row is formed once, by one warp, for half of what that
+// costs (16 blocks 72 -> 80 us).
 __device__ __forceinline__ Z zinv(Z p, int *bad) {
     const double t = p.y / p.x, den = fma(p.y, t, p.x);  // 1/p = (1 - i t) / (p.x + p.y t), p.y ~ 0 here
     if (!(p.x > 0.0) || !isfinite(p.x * p.x + p.y * p.y)) *bad = 1;       // not positive definite
@@ -112,7 +117,7 @@ __device__ __forceinline__ Z zinv(Z p, int *bad) {
 }
 
 __global__ void __launch_bounds__(256) k6_diag(double2 *__restrict__ A, int n, int k0, int kb, int *err) {
-    __shared__ Z row[2][kB], col[2][kB], pivinv[2];
+    __shared__ Z row[2][kB], col[2][kB], pivinv[2], scaled[kB];
     __shared__ int bad[2];       // of the current and the next pivot: never written while it is read
     const long j = blockIdx.x;
     double2 *M = A + j * (long)n * n;
@@ -141,12 +146,11 @@ __global__ void __launch_bounds__(256) k6_diag(double2 *__restrict__ A, int n, i
             return;
         }
         // row k scaled, g = a_k. / p, and the multipliers -a_.k of this thread's rows
+        if (threadIdx.x < kB) scaled[threadIdx.x] = threadIdx.x == k ? p : zmul(row[cur][threadIdx.x], p);
+        __syncthreads();
         Z g[2], f[2];
 #pragma unroll
-        for (int l = 0; l < 2; ++l) {
-            const int c = c0 + 16 * l;
-            g[l] = c == k ? p : zmul(row[cur][c], p);
-        }
+        for (int l = 0; l < 2; ++l) g[l] = scaled[c0 + 16 * l];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             f[i] = col[cur][r0 + 16 * i];
@@ -158,7 +162,8 @@ __global__ void __launch_bounds__(256) k6_diag(double2 *__restrict__ A, int n, i
             for (int l = 0; l < 2; ++l) {
                 const int r = r0 + 16 * i, c = c0 + 16 * l;
                 Z v = c == k ? Z{0.0, 0.0} : a[i][l];       // column k becomes -a_rk / p
-                v = r == k ? g[l] : zfma(f[i], g[l], v);
+                const Z t = zmul(f[i], g[l]);
+                v = r == k ? g[l] : Z{v.x + t.x, v.y + t.y};
                 a[i][l] = v;
                 if (r == k + 1) row[nxt][c] = v;
                 if (c == k + 1) col[nxt][r] = v;
