@@ -730,7 +730,7 @@ def unfold_measure(B, torch, p, dev_in, stream, reps=3):
     gbs = nbytes / (ms * 1e-3) / 1e9
     hbm = measured_hbm_gbs()
     del cin, cout
-    return {"what": "c(G) -> U c(R^-1 G) e^{-iG.tau} (FP64), one launch over the bands of the step's "
+    return {"what": "c(G) -> U c(R^-1 G) e^{-iG.tau} (FP64), one call for the bands of the step's "
                     "k-points (at most 16384) on the sphere of k-point 0",
             "bands": nb, "plane_waves": ngw, "bytes": nbytes, "ms": ms, "gbs": gbs, "peak_gbs": hbm,
             "hbm_frac": gbs / hbm if hbm else None,
